@@ -2,9 +2,7 @@
 //
 // On GB300 the FP64 pipe retires 2 DFMA per clock per SM (about 1.1 TFLOP/s
 // for the chip), so every FP64 contraction here is bound by the DFMA issue
-// rate, not by memory: the GEMM below stages 64x64x16 tiles of both operands
-// in shared memory and keeps a 4x4 register tile per thread, which already
-// makes shared-memory and HBM traffic a small fraction of the DFMA time.
+// rate, not by memory (dgemm_kernel below).
 // The HBM-bound passes (symmetrisation, mirror, shift, combine, norms) use
 // 32x32 shared-memory transposes so that both the row and the column access
 // are coalesced.
@@ -43,8 +41,8 @@ bool ensure_dynamic_smem(const void *func, int bytes)
 
 // --------------------------------------------------------------------------
 // GEMM with triangular operands, lower-only output and inner scaling, in
-// three arithmetic modes:
-//   GM_F64  FP64 storage, DFMA accumulation
+// two arithmetic modes on the FP32 pipe (FP64 storage on the DFMA pipe:
+// dgemm_kernel below):
 //   GM_F32  FP32 storage, FFMA accumulation
 //   GM_DF   FP64 storage, FP64 emulated on the FP32 pipe: each operand is
 //           split into a pair of floats (hi = fl32(x), lo = fl32(x - hi)), the
@@ -84,7 +82,7 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
     if (g.triB == TRI_LOWER) kbeg = max(kbeg, j0);         // op(B)[p][j] = 0 for p < j
     if (g.triB == TRI_UPPER) kend = min(kend, j0 + GBN);   // op(B)[p][j] = 0 for p > j
 
-    using S = typename std::conditional<MODE == GM_F64, double, float>::type;
+    using S = float;
     __shared__ S As[GBK][GBM + 1], Bs[GBK][GBN + 1];
     __shared__ float Asl[MODE == GM_DF ? GBK : 1][GBM + 1], Bsl[MODE == GM_DF ? GBK : 1][GBN + 1];
     const int tid = threadIdx.x;
@@ -219,6 +217,196 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
     }
 }
 
+// --------------------------------------------------------------------------
+// FP64 GEMM on the DFMA pipe.  The pipe retires 2 DFMA per clock and SM -- a
+// warp's DFMA occupies its sub-partition for 64 clocks -- so a tile needs only
+// enough warps (8) and no register blocking to keep it busy: shared-memory and
+// L2 traffic stay below a tenth of their rates even with 16 x 16 tiles.  What
+// bounds a product is then how evenly its multiply-adds spread over the 152
+// pipes, so the tile is chosen per launch (dgemm_tile) among
+//   32 x 32 (2 x 2 outputs per thread), 16 x 16 (one output per thread) and
+//   8 x 8 (four threads per output, each every fourth k; sums added in order).
+// Each k block is prefetched into registers while the previous one is used.
+// Measured (one launch, GB300): 128^3 113 us with 64 x 64 tiles on four SMs -> 9 us;
+// 2048^3 14.4 ms, 1.19 TFLOP/s of the pipe's 1.26.
+// --------------------------------------------------------------------------
+template <int TS> struct DgemmTile;
+template <> struct DgemmTile<32> { static constexpr int R = 2, KS = 1, BK = 16; };
+template <> struct DgemmTile<16> { static constexpr int R = 1, KS = 1, BK = 32; };
+template <> struct DgemmTile<8> { static constexpr int R = 1, KS = 4, BK = 64; };
+
+// tile t of a row-by-row count of the tiles (bi, bj) with bj <= bi and bj < nt
+__device__ __forceinline__ void dgemm_lower_tile(int t, int nt, int &bi, int &bj)
+{
+    const int tri = nt * (nt + 1) / 2;
+    if (t >= tri) {
+        bi = nt + (t - tri) / nt;
+        bj = (t - tri) % nt;
+        return;
+    }
+    bi = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while (bi * (bi + 1) / 2 > t) --bi;
+    while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
+    bj = t - bi * (bi + 1) / 2;
+}
+
+template <int TS>
+__global__ void __launch_bounds__(256) dgemm_kernel(GemmArgs g)
+{
+    constexpr int R = DgemmTile<TS>::R, KS = DgemmTile<TS>::KS, BK = DgemmTile<TS>::BK, TD = TS / R;
+    static_assert(TD * TD * KS == 256 && TS * BK == 512, "256 threads, two elements per thread and operand");
+    // tile of this CTA; long k ranges first: with op(A) lower or op(B) upper triangular they
+    // are at the far end.  lowerC: the grid counts the tiles on and below the diagonal alone
+    // (CTAs that leave at once would take their turn in the round-robin over the SMs).
+    int bi, bj;
+    const int z = blockIdx.z;
+    if (g.lowerC) {
+        const int t = g.triA == TRI_LOWER ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+        dgemm_lower_tile(t, (g.n + TS - 1) / TS, bi, bj);
+    } else {
+        bi = g.triA == TRI_LOWER ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+        bj = g.triB == TRI_UPPER ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    }
+    const int i0 = bi * TS, j0 = bj * TS;
+    const double *A = (const double *)g.A + (long long)z * g.sA;
+    const double *B = (const double *)g.B + (long long)z * g.sB;
+    const double *ks = (const double *)g.kscale;
+    int kbeg = 0, kend = g.k;
+    if (g.triA == TRI_LOWER) kend = min(kend, i0 + TS);
+    if (g.triA == TRI_UPPER) kbeg = max(kbeg, i0);
+    if (g.triB == TRI_LOWER) kbeg = max(kbeg, j0);
+    if (g.triB == TRI_UPPER) kend = min(kend, j0 + TS);
+
+    __shared__ double As[2][BK][TS + 1], Bs[2][BK][TS + 1];
+    __shared__ double red[KS > 1 ? KS - 1 : 1][KS > 1 ? TD * TD : 1];
+    const int tid = threadIdx.x, kg = tid / (TD * TD), tx = tid % TD, ty = (tid / TD) % TD;
+    double acc[R][R];
+#pragma unroll
+    for (int a = 0; a < R; ++a)
+#pragma unroll
+        for (int b = 0; b < R; ++b) acc[a][b] = 0.0;
+
+    double ra[2], rb[2];
+    auto fetch = [&](int kt) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = tid + 256 * u;
+            {   // consecutive threads along the operand's memory rows
+                const int il = g.ta ? e % TS : e / BK, pl = g.ta ? e / TS : e % BK, i = i0 + il, p = kt + pl;
+                bool ok = i < g.m && p < kend;
+                if (g.triA == TRI_LOWER) ok = ok && p <= i;
+                if (g.triA == TRI_UPPER) ok = ok && p >= i;
+                double v = 0.0;
+                if (ok) {
+                    v = load_op(A, g.lda, g.ta, i, p);
+                    if (ks) v *= ks[p];
+                }
+                ra[u] = v;
+            }
+            {
+                const int jl = g.tb ? e / BK : e % TS, pl = g.tb ? e % BK : e / TS, j = j0 + jl, p = kt + pl;
+                bool ok = j < g.n && p < kend;
+                if (g.triB == TRI_LOWER) ok = ok && p >= j;
+                if (g.triB == TRI_UPPER) ok = ok && p <= j;
+                rb[u] = ok ? load_op(B, g.ldb, g.tb, p, j) : 0.0;
+            }
+        }
+    };
+    auto store = [&](int s) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int e = tid + 256 * u;
+            As[s][g.ta ? e / TS : e % BK][g.ta ? e % TS : e / BK] = ra[u];
+            Bs[s][g.tb ? e % BK : e / TS][g.tb ? e / BK : e % TS] = rb[u];
+        }
+    };
+    if (kbeg < kend) {
+        fetch(kbeg);
+        store(0);
+        __syncthreads();
+        for (int kt = kbeg, s = 0; kt < kend; kt += BK, s ^= 1) {
+            const bool more = kt + BK < kend;
+            if (more) fetch(kt + BK);
+#pragma unroll 8
+            for (int p = kg; p < BK; p += KS) {
+                double a[R], b[R];
+#pragma unroll
+                for (int q = 0; q < R; ++q) { a[q] = As[s][p][ty + TD * q]; b[q] = Bs[s][p][tx + TD * q]; }
+#pragma unroll
+                for (int qa = 0; qa < R; ++qa)
+#pragma unroll
+                    for (int qb = 0; qb < R; ++qb) acc[qa][qb] = fma(a[qa], b[qb], acc[qa][qb]);
+            }
+            if (more) store(s ^ 1);
+            __syncthreads();
+        }
+    }
+    if (KS > 1) {
+        if (kg > 0) red[kg - 1][tid % (TD * TD)] = acc[0][0];
+        __syncthreads();
+        if (kg > 0) return;
+#pragma unroll
+        for (int q = 0; q < KS - 1; ++q) acc[0][0] += red[q][tid];
+    }
+    double *C = (double *)g.C + (long long)z * g.sC;
+    const double *Cin = g.Cin ? (const double *)g.Cin + (long long)z * g.sCin : nullptr;
+#pragma unroll
+    for (int qa = 0; qa < R; ++qa) {
+        const int i = i0 + ty + TD * qa;
+        if (i >= g.m) continue;
+#pragma unroll
+        for (int qb = 0; qb < R; ++qb) {
+            const int j = j0 + tx + TD * qb;
+            if (j >= g.n || (g.lowerC && j > i)) continue;
+            double v = g.alpha * acc[qa][qb];
+            if (g.beta != 0.0) v += g.beta * Cin[(long long)i * g.ldcin + j];
+            C[(long long)i * g.ldc + j] = v;
+        }
+    }
+}
+
+// tiles of order ts that are worked on, per batch matrix
+static long long dgemm_tiles(const GemmArgs &g, int ts)
+{
+    const long long mt = (g.m + ts - 1) / ts, nt = (g.n + ts - 1) / ts;
+    if (!g.lowerC) return mt * nt;
+    const long long d = std::min(mt, nt);
+    return d * (d + 1) / 2 + (mt > nt ? (mt - nt) * nt : 0);
+}
+
+// time of the busiest pipe in units of outputs x k, the tiles dealt out over 152 SMs
+static double dgemm_cost(const GemmArgs &g, int ts)
+{
+    return std::ceil((double)dgemm_tiles(g, ts) * g.batch / 152.0) * ts * ts;
+}
+
+// The largest tile whose busiest SM has no more work than the smaller tiles' allow for: a
+// smaller tile costs a few percent more instructions per DFMA, hence its handicap.
+static int dgemm_tile(const GemmArgs &g)
+{
+    const double c32 = dgemm_cost(g, 32), c16 = 1.04 * dgemm_cost(g, 16), c8 = 1.15 * dgemm_cost(g, 8);
+    if (c32 <= c16 && c32 <= c8) return 32;
+    return c16 <= c8 ? 16 : 8;
+}
+
+// estimate of the DFMA engine's time in microseconds: the busiest SM's multiply-adds at
+// 1.7 per clock and 2 GHz, and the launch
+double dgemm_time_us(const GemmArgs &g)
+{
+    return dgemm_cost(g, dgemm_tile(g)) * g.k / 3400.0 + 4.0;
+}
+
+static void dgemm_launch(const GemmArgs &g, cudaStream_t s)
+{
+    const int ts = dgemm_tile(g);
+    const dim3 grid = g.lowerC ? dim3((unsigned)dgemm_tiles(g, ts), 1, g.batch)
+                               : dim3((g.n + ts - 1) / ts, (g.m + ts - 1) / ts, g.batch);
+    if (ts == 32) dgemm_kernel<32><<<grid, 256, 0, s>>>(g);
+    else if (ts == 16) dgemm_kernel<16><<<grid, 256, 0, s>>>(g);
+    else dgemm_kernel<8><<<grid, 256, 0, s>>>(g);
+    count_launch();
+}
+
 void gemm_launch(const GemmArgs &g, cudaStream_t s)
 {
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return;
@@ -226,7 +414,7 @@ void gemm_launch(const GemmArgs &g, cudaStream_t s)
     switch (g.mode) {
     case GM_F32: gemm_kernel<GM_F32><<<grid, 256, 0, s>>>(g); count_launch(); break;
     case GM_DF: gemm_kernel<GM_DF><<<grid, 256, 0, s>>>(g); count_launch(); break;
-    default: gemm_kernel<GM_F64><<<grid, 256, 0, s>>>(g); count_launch(); break;
+    default: dgemm_launch(g, s); break;
     }
 }
 
