@@ -664,6 +664,14 @@ int oz_gemm_run(const GemmArgs &g, void *ws, int *err, cudaStream_t s)
     return 0;
 }
 
+// estimate of the slice engine's time in microseconds: the four launches, prologue and
+// epilogue, then the k blocks of the tiles a busiest SM takes in turn
+double oz_gemm_time_us(const GemmArgs &g)
+{
+    const double mt = (g.m + OZ_BM - 1) / OZ_BM, nt = (g.n + OZ_BN - 1) / OZ_BN;
+    return 30.0 + std::ceil((g.lowerC ? 0.5 : 1.0) * mt * nt * g.batch / 152.0) * (g.k / OZ_BK) * 0.56;
+}
+
 int oz_gemm_launch(const GemmArgs &g, void *ws, int *err, cudaStream_t s)
 {
     int st = oz_gemm_prepare(g, ws, s);

@@ -65,6 +65,7 @@ struct pssd_handle_s {
     int *derr = nullptr;    // device error flag of the current call (bounded waits in the tensor-core kernel)
     int use_tc = 1;         // FP32 contractions on tcgen05 tensor cores (0: FP32 SIMT kernel)
     int force_engine = 0;   // test hooks: no size-based engine selection
+    bool pinned = false;    // products upstream of the mixed mode's FP32 stage (see gemm())
     bool user_ws = false;   // chunks[0] is caller-owned memory (pssd_set_workspace); never allocate
     size_t depth = 0;       // bytes of workspace live in the current call (stack discipline)
     size_t peak = 0;        // largest depth reached since creation or pssd_set_workspace
@@ -273,10 +274,19 @@ void gemm(pssd_handle h, const GemmArgs &g0)
     double fl = h->prof ? 2.0 * gemm_macs(g) : 0.0;
     Mark mk = mark(h);
     if (g.mode == GM_OZ && !h->derr) g.mode = GM_DF;   // (no error flag outside a guarded call)
-    // very thin or tiny products: the slicing passes would dominate; use float pairs
-    // (the slices are FP64-accurate, the float pairs carry ~2^-47 per product)
-    if (g.mode == GM_OZ && !h->force_engine && (g.k < 16 || (double)g.m * g.n * g.k * g.batch < 262144.0))
-        g.mode = GM_DF;
+    // Small products: the slice engine's four launches and its tile latency dominate, and the
+    // FP64 pipes finish first (64^3: 5 us against 28 us; 256^3: 38 us against 44 us; 384^3: 115 us
+    // against 50 us, so the estimates decide).  Upstream of the mixed mode's FP32 iteration the
+    // engines are pinned -- float pairs for thin or tiny products, slices for the rest: the
+    // iteration turns a flipped last bit of its input into a change of the size of its own
+    // error, so mixed results would otherwise move with every choice made here.
+    if (g.mode == GM_OZ && !h->force_engine) {
+        if (h->pinned) {
+            if (g.k < 16 || (double)g.m * g.n * g.k * g.batch < 262144.0) g.mode = GM_DF;
+        } else if (dgemm_time_us(g) <= oz_gemm_time_us(g)) {
+            g.mode = GM_F64;
+        }
+    }
     if (g.mode == GM_DF) {
         // split each FP64 operand into compact float pairs once (stream-ordered temporaries)
         const int ra = g.ta ? g.k : g.m, cla = g.ta ? g.m : g.k;
@@ -1623,6 +1633,7 @@ int front(pssd_handle h, int n, const signed char *sigma, const double *H, int l
     // keep the shifted inverses of every step, else only the per-step iterates
     PhaseScope phase(PH_FRONT);
     F.n = n;
+    h->pinned = o.precision == PSSD_MIXED;   // until the FP32 stage has its input
     h->wait_limit = o.wait_cycles;
     if (info) info->method = o.method;
     h->use_tc = (o.flags & PSSD_FLAG_NO_TENSOR_CORES) ? 0 : 1;
@@ -1685,6 +1696,7 @@ int front(pssd_handle h, int n, const signed char *sigma, const double *H, int l
         gemm(h, b);                                                      // L^T S L^{-T} (symmetric; lower, mirrored)
         mirror(h, F.Y, ld, 0, n, 1);
         release(h, mk);
+        h->pinned = false;
         return PSSD_OK;
     }
     // a3: bounds (reading R5: |lambda(H)| in [lambda_min(M), lambda_max(M)])
@@ -1732,6 +1744,7 @@ int front(pssd_handle h, int n, const signed char *sigma, const double *H, int l
             Timed t(h, K_HBM, 0, 12.0 * n * (double)n);
             scale_copy<double, float>(F.K, ld, X32, ld, n, n, 1.0 / alpha, h->stream);
         }
+        h->pinned = false;
         float *Y32 = nullptr;
         int st = zolo_sign_fp32(h, X32, n, beta / alpha, 1e-6, 3e-3, fA, fB, &Y32, info, &fi);
         if (st) { if (info) info->fail_index = fi; release(h, mk); return st; }
@@ -1817,6 +1830,7 @@ int guarded(pssd_handle h, pssd_info *info, F body)
     Mark mk = mark(h);
     int st;
     h->wait_limit = 0;   // the default bound unless the call's options set one (front())
+    h->pinned = false;
     int *outer_err = h->derr;
     try {
         if (!outer_err) {

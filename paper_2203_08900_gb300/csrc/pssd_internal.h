@@ -75,6 +75,7 @@ struct GemmArgs {
 void split_pairs(const double *x, long long ld, long long sb, int rows, int cols, int batch, float *hi, float *lo,
                  cudaStream_t s);
 void gemm_launch(const GemmArgs &g, cudaStream_t s);
+double dgemm_time_us(const GemmArgs &g);   // estimated time of GM_F64 (chooses between the FP64-accurate engines)
 // FP32 GEMM on tcgen05 tensor cores (3xTF32), same conventions as GM_F32;
 // ws: tc_gemm_workspace_bytes(g) bytes of device memory; err: device flag.
 size_t tc_gemm_workspace_bytes(const GemmArgs &g);
@@ -87,6 +88,7 @@ size_t oz_gemm_workspace_bytes(const GemmArgs &g);
 int oz_gemm_launch(const GemmArgs &g, void *ws, int *err, cudaStream_t s);
 int oz_gemm_prepare(const GemmArgs &g, void *ws, cudaStream_t s);           // exponent and slicing passes only
 int oz_gemm_run(const GemmArgs &g, void *ws, int *err, cudaStream_t s);     // product on prepared slices
+double oz_gemm_time_us(const GemmArgs &g);   // estimated time of both
 
 // Cholesky and triangular inverse of the s x s diagonal block at (off, off)
 // of each batch matrix, in one launch: L (lower) in place in A with zeros
