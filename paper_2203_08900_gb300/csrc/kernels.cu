@@ -391,10 +391,10 @@ static int dgemm_tile(const GemmArgs &g)
 }
 
 // estimate of the DFMA engine's time in microseconds: the busiest SM's multiply-adds at
-// 1.7 per clock and 2 GHz, and the launch
+// 2 per clock and 2 GHz, and the launch
 double dgemm_time_us(const GemmArgs &g)
 {
-    return dgemm_cost(g, dgemm_tile(g)) * g.k / 3400.0 + 4.0;
+    return dgemm_cost(g, dgemm_tile(g)) * g.k / 4000.0 + 4.0;
 }
 
 static void dgemm_launch(const GemmArgs &g, cudaStream_t s)

@@ -28,11 +28,19 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// bounded wait for the phase with the given parity; false on timeout
+// Bounded wait for the phase with the given parity; false on timeout.  The first poll returns at
+// once; the later ones may be suspended for a while by the hardware.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit)
 {
-    for (unsigned long long it = 0; it < limit; ++it) {
-        uint32_t done;
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    for (unsigned long long it = 1; !done && it < limit; ++it)
         asm volatile(
             "{\n.reg .pred p;\n"
             "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
@@ -40,9 +48,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
             : "=r"(done)
             : "r"(bar), "r"(parity)
             : "memory");
-        if (done) return true;
-    }
-    return false;
+    return done != 0;
 }
 
 }  // namespace pssd

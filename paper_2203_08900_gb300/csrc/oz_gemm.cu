@@ -47,6 +47,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -76,7 +77,8 @@ constexpr int OZ_GROUP_M = 8;              // row blocks per group of the tile o
 
 struct OzArgs {
     // slices, tiled: block (z, row tile, k block) = 8 slices x tile rows x 16 k,
-    // 32-byte-swizzled rows, contiguous (32 KB for A, 16 KB for B)
+    // 32-byte-swizzled rows, contiguous (32 KB for A, 16 KB for B): one copy per operand and k
+    // block (with one copy per slice, 16 in all, a 4096^3 product took 3.32 ms instead of 2.73)
     const __nv_bfloat16 *sa, *sb;
     int kblocks;                           // k_pad / 16
     int m, n, k, batch, m_pad, n_pad;
@@ -116,18 +118,33 @@ __host__ __device__ constexpr uint32_t oz_idesc(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(OZ_BM >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, unsigned long long a, unsigned long long b, uint32_t idesc,
-                                         uint32_t acc)
+// one product of stacked slices; the descriptors' low words and their common high word
+__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t dhi, uint32_t idesc,
+                                         uint32_t acc, uint32_t pred)
 {
     asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+        "{\n.reg .pred p, q;\n.reg .b64 da, db;\n"
+        "setp.ne.b32 p, %5, 0;\nsetp.ne.b32 q, %6, 0;\n"
+        "mov.b64 da, {%1, %3};\nmov.b64 db, {%2, %3};\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(tmem_d),
+        "r"(alo), "r"(blo), "r"(dhi), "r"(idesc), "r"(acc), "r"(pred));
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t bar)
+__device__ __forceinline__ void mma_commit_if(uint32_t bar, uint32_t pred)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+        "r"(pred)
+        : "memory");
+}
+
+// 1 in one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+    return e;
 }
 
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t *r)
@@ -247,43 +264,47 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
         }
     } else if (warp == OZ_MMA_WARP) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            for (int c = 0; c < nchunks && !s_abort; ++c) {
-                if (c > 0 && !mbar_wait(b_free, (uint32_t)((c - 1) & 1), g.wait_limit)) {
-                    s_abort = 1; atomicExch(g.err, 2); break;
-                }
+        // The warp runs converged and one elected lane issues, so that the operands stay in
+        // uniform registers: from a lane in a branch of its own a k block took 1500 clocks to
+        // issue, more than its 36 products (1152).
+        const uint32_t leader = elect_one();
+        const uint32_t dhi = (uint32_t)(smem_desc_sw32(0) >> 32), dlo0 = (uint32_t)smem_desc_sw32(smem_u32(smem));
+        bool ok = true;
+        int s = 0;
+        uint32_t phase = 0;
+        for (int c = 0; c < nchunks && ok; ++c) {
+            if (c > 0 && !mbar_wait(b_free, (uint32_t)((c - 1) & 1), g.wait_limit)) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const int q0 = c * OZ_CHUNK_STAGES, q1 = min(nkb, q0 + OZ_CHUNK_STAGES);
+#pragma unroll 1
+            for (int q = q0; q < q1; ++q) {
+                if (!mbar_wait(b_full + 8 * s, phase, g.wait_limit)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;");
-                const int q0 = c * OZ_CHUNK_STAGES, q1 = min(nkb, q0 + OZ_CHUNK_STAGES);
-                bool ok = true;
-                for (int q = q0; q < q1; ++q) {
-                    const int s = q % OZ_STAGES;
-                    if (!mbar_wait(b_full + 8 * s, (uint32_t)((q / OZ_STAGES) & 1), g.wait_limit)) { ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;");
-                    const uint32_t st = smem_u32(smem + s * OZ_STAGE_BYTES);
-                    // A slice a against B slices b = 1 .. S+1-a stacked along N: the product
-                    // (a, b) belongs to level a+b-2, whose accumulator starts at column
-                    // 64 (a+b-2), so slices b..b+3 form one N <= 256 MMA into consecutive levels.
+                const uint32_t dlo = dlo0 + (uint32_t)(s * (OZ_STAGE_BYTES >> 4));
+                const uint32_t fresh = q == q0 ? 0u : 1u;   // a = 1 reaches every level first
+                // A slice a against B slices b = 1 .. S+1-a stacked along N: the product
+                // (a, b) belongs to level a+b-2, whose accumulator starts at column
+                // 64 (a+b-2), so slices b..b+3 form one N <= 256 MMA into consecutive levels.
 #pragma unroll
-                    for (int a = 1; a <= OZ_S; ++a) {
-                        const unsigned long long ad = smem_desc_sw32(st + (a - 1) * OZ_A_TILE);
-                        const uint32_t acc = (q == q0 && a == 1) ? 0u : 1u;   // a = 1 reaches every level first
+                for (int a = 1; a <= OZ_S; ++a) {
 #pragma unroll
-                        for (int b0 = 1; b0 <= OZ_S + 1 - a; b0 += 4) {
-                            const int nb = min(4, OZ_S + 2 - a - b0);
-                            const unsigned long long bd = smem_desc_sw32(st + OZ_S * OZ_A_TILE + (b0 - 1) * OZ_B_TILE);
-                            mma_bf16(tmem + (uint32_t)((a + b0 - 2) * OZ_BN), ad, bd, oz_idesc(nb * OZ_BN), acc);
-                        }
+                    for (int b0 = 1; b0 <= OZ_S + 1 - a; b0 += 4) {
+                        const int nb = min(4, OZ_S + 2 - a - b0);
+                        mma_bf16(tmem + (uint32_t)((a + b0 - 2) * OZ_BN), dlo + (uint32_t)((a - 1) * OZ_A_TILE >> 4),
+                                 dlo + (uint32_t)((OZ_S * OZ_A_TILE + (b0 - 1) * OZ_B_TILE) >> 4), dhi,
+                                 oz_idesc(nb * OZ_BN), a == 1 ? fresh : 1u, leader);
                     }
-                    mma_commit(b_empty + 8 * s);
                 }
-                if (!ok) { s_abort = 1; atomicExch(g.err, 3); break; }
-                mma_commit(b_done);
+                mma_commit_if(b_empty + 8 * s, leader);
+                if (++s == OZ_STAGES) { s = 0; phase ^= 1; }
             }
-            // Every MMA issued has retired before TMEM and the stages go away, whatever
-            // the other roles did (a flush warp that gave up no longer waits for them).
-            mma_commit(b_drain);
-            mbar_wait(b_drain, 0u, OZ_WAIT_LIMIT);
+            if (ok) mma_commit_if(b_done, leader);
         }
+        if (!ok && leader) { s_abort = 1; atomicExch(g.err, 2); }
+        // Every MMA issued has retired before TMEM and the stages go away, whatever
+        // the other roles did (a flush warp that gave up no longer waits for them).
+        mma_commit_if(b_drain, leader);
+        mbar_wait(b_drain, 0u, OZ_WAIT_LIMIT);
     } else {
         // ---------------- flush warps: lanes 32 (w % 4) .., columns c0 .. c0 + 15 ----------------
         const int quad = warp & 3, c0 = (warp >> 2) * OZ_FCOLS;
@@ -346,17 +367,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
 //   logical operand X(r, p), r < rows, p < k:  trans ? src[p][r] : src[r][p],
 //   structural zeros (tri, in (r, p) terms) forced to 0, optional ks[p] scaling
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double oz_load(const double *X, long long ld, int trans, int rows, int k, int tri,
-                                          const double *ks, int r, int p)
-{
-    if (r >= rows || p >= k) return 0.0;
-    if (tri == TRI_LOWER && p > r) return 0.0;
-    if (tri == TRI_UPPER && p < r) return 0.0;
-    double v = trans ? X[(long long)p * ld + r] : X[(long long)r * ld + p];
-    if (ks) v *= ks[p];
-    return v;
-}
-
 // frexp exponent of v (v = f 2^e, 0.5 <= |f| < 1) from the IEEE-754 fields;
 // a very small value for zero
 __device__ __forceinline__ int oz_frexp_exp(double v)
@@ -418,154 +428,120 @@ __device__ __forceinline__ void oz_digits(long long F, uint32_t *bits)
     bits[0] = oz_small_int_bits(hi);
 }
 
-// One operand of the preparation passes: op(X) is rows x k (trans: op(X)[r][p] = X[p][r]),
-// with structural zeros (tri), an optional inner scaling ks[p], rows padded to rows_pad.
+// One operand of the preparation: op(X) is rows x k (trans: op(X)[r][p] = X[p][r]), with
+// structural zeros (tri), an optional inner scaling ks[p], rows padded to rows_pad.
 struct OzOperand {
     const double *X; long long ld, sb; int trans, rows, tri; const double *ks;
     int rows_pad, tile_rows; int *e; __nv_bfloat16 *out;
 };
 
-// exponents e(r) with max_p |op(X)[r][p]| < 2^e of both operands in one launch; blocks
-// [0, nA) serve A, the rest B.  Rows contiguous in memory (trans = 0): a block holds 8 warps,
-// each one row over a 1024-column chunk (8 loads in flight per lane), a shuffle max and an
-// atomicMax.  Transposed (trans = 1): a block covers 32 rows of op(X) (32 memory columns)
-// over a 256-term chunk of p, its 8 warps each reading 32 p rows of 32 consecutive doubles,
-// then a shared-memory max and one atomicMax per row.
-__global__ void __launch_bounds__(256) oz_exp_kernel(OzOperand a, OzOperand b, int k, int nA)
+// Exponents and slices of both operands in one launch; blocks [0, nA) serve A, the rest B.  A
+// CTA has a band of 16 rows of op(X) and all of k: it reads the band for the rows' largest
+// magnitudes, then again -- 128 KB at k = 1024, from L2 -- for the digits.  A warp covers the 16
+// rows of one k block (16 columns); a lane has eight consecutive columns of one row, and each of
+// its slices is one 16-byte store, 512 contiguous bytes per warp.  With trans = 0 the two lanes
+// of a row read 128 contiguous bytes between them, with trans = 1 half a warp reads 16
+// consecutive doubles of a memory row: no transposition through shared memory.  Bound by HBM:
+// 8 B read and 16 B written per element (4096^2, both operands: 200 us in one launch; three
+// launches took 303 us: a fill, an exponent pass over the matrix, the slices).
+// F = round(x 2^{56-e}) is cut into balanced base-128 digits: x 2^{-e} = sum_t d_t 2^{-7t} +
+// O(2^-57).  In shared memory the GEMM expects 32-byte rows whose 16-byte halves are swapped where bit 2 of the row
+// is set (the 32-byte swizzle), so they are written that way.
+__global__ void __launch_bounds__(256) oz_prepare_kernel(OzOperand a, OzOperand b, int k, int k_pad, int nA)
 {
+    __shared__ int top[8][16];
     const bool isA = (int)blockIdx.x < nA;
     const OzOperand &o = isA ? a : b;
-    const int blk = isA ? (int)blockIdx.x : (int)blockIdx.x - nA;
-    const int z = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int z = blockIdx.z, r0 = (isA ? (int)blockIdx.x : (int)blockIdx.x - nA) * 16;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // rows next to each other in memory go to lanes next to each other
+    const int rl = o.trans ? lane & 15 : lane >> 1, half = o.trans ? lane >> 4 : lane & 1;
+    const int r = r0 + rl, kblocks = k_pad / 16;
     const double *X = o.X + (long long)z * o.sb;
-    if (!o.trans) {
-        const int kc = (k + 1023) / 1024;                  // chunks per row
-        const int r = (blk / kc) * 8 + warp, p0 = (blk % kc) * 1024;
-        if (r >= o.rows) return;
-        int mx = INT_MIN / 2;
-        for (int pp = p0; pp < p0 + 1024 && pp < k; pp += 256) {
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-                mx = max(mx, oz_frexp_exp(oz_load(X, o.ld, 0, o.rows, k, o.tri, o.ks, r, pp + t * 32 + lane)));
-        }
-#pragma unroll
-        for (int q = 16; q > 0; q >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, q));
-        if (lane == 0 && mx > INT_MIN / 2) atomicMax(&o.e[z * o.rows_pad + r], mx);
-    } else {
-        __shared__ int red[8][33];
-        const int kc = (k + 255) / 256;
-        const int r0 = (blk / kc) * 32, p0 = (blk % kc) * 256;
-        const int r = r0 + lane;
-        int mx = INT_MIN / 2;
-#pragma unroll 4
-        for (int t = 0; t < 32; ++t) {
-            const int pp = p0 + warp + 8 * t;
-            mx = max(mx, oz_frexp_exp(oz_load(X, o.ld, 1, o.rows, k, o.tri, o.ks, r, pp)));
-        }
-        red[warp][lane] = mx;
-        __syncthreads();
-        if (warp == 0) {
-#pragma unroll
-            for (int w = 1; w < 8; ++w) mx = max(mx, red[w][lane]);
-            if (r < o.rows && mx > INT_MIN / 2) atomicMax(&o.e[z * o.rows_pad + r], mx);
-        }
-    }
-}
-
-// number of blocks oz_exp_kernel uses for one operand
-int oz_exp_blocks(const OzOperand &o, int k)
-{
-    if (!o.trans) return ((o.rows + 7) / 8) * ((k + 1023) / 1024);
-    return ((o.rows + 31) / 32) * ((k + 255) / 256);
-}
-
-// eight BF16 slices in the tiled layout the GEMM streams: for row r of tile
-// rr = r % tile_rows and column p (k block p / 16, kk = p % 16) of slice t the
-// element sits in block ((z * rows_pad / tile_rows + r / tile_rows) * kblocks + p / 16)
-// of 8 * tile_rows * 16 elements, at t * tile_rows * 16 + rr * 16 + kk with the
-// 16-byte half of the 32-byte row flipped when bit 2 of rr is set (the 32-byte
-// shared-memory swizzle the MMA descriptors expect).
-// F = round(x 2^{56-e}) is cut into balanced base-128 digits d_8 .. d_2 in
-// [-64, 63]; the rest is d_1, |d_1| <= 128; x 2^{-e} = sum_t d_t 2^{-7t} + O(2^-57).
-// One CTA per 32 rows x 64 columns of op(X): the tile is read coalesced (along memory
-// rows, transposing through shared memory when trans = 1), then each thread takes 8
-// consecutive columns of one row -- half of a 16-column k block -- and writes each of
-// its 8 slices as one 16-byte store; the 32 lanes of a warp cover 16 rows x both halves
-// of one k block, i.e. 512 contiguous bytes per slice.
-__global__ void __launch_bounds__(256) oz_slice_kernel(OzOperand a, OzOperand b, int k, int k_pad, int nA)
-{
-    __shared__ double T[32][65];               // T[row][column] of the tile
-    const bool isA = (int)blockIdx.x < nA;
-    const OzOperand &o = isA ? a : b;
-    const int blk = isA ? (int)blockIdx.x : (int)blockIdx.x - nA;
-    const int pt = (k_pad + 63) / 64;           // 64-column tiles per row band
-    const int z = blockIdx.z, r0 = (blk / pt) * 32, p0 = (blk % pt) * 64;
-    const int tid = threadIdx.x;
-    const double *X = o.X + (long long)z * o.sb;
-    const int trans = o.trans, rows = o.rows, tri = o.tri, rows_pad = o.rows_pad, tile_rows = o.tile_rows;
     const long long ld = o.ld;
-    const double *ks = o.ks;
-    const int *e = o.e;
-    __nv_bfloat16 *out = o.out;
-    if (trans) {   // memory rows are p: a warp reads 32 consecutive r of one p
-        for (int it = 0; it < 8; ++it) {
-            const int pl = it * 8 + (tid >> 5), rl = tid & 31;
-            T[rl][pl] = oz_load(X, ld, 1, rows, k, tri, ks, r0 + rl, p0 + pl);
+    const bool live = r < o.rows;
+    // columns of this row that are not structurally zero
+    const int plo = o.tri == TRI_UPPER ? r : 0, phi = o.tri == TRI_LOWER ? min(k, r + 1) : k;
+    // k blocks that hold any of the band's columns
+    const int kb_lo = o.tri == TRI_UPPER ? min(r0 / 16, kblocks) : 0;
+    const int kb_hi = o.tri == TRI_LOWER ? min(kblocks, r0 / 16 + 1) : kblocks;
+    const bool quads = !o.trans && (ld & 1) == 0 && ((uintptr_t)X & 15) == 0;
+    auto load = [&](int kb, double *v) {
+        const int p0 = kb * 16 + half * 8;
+        const bool whole = live && p0 >= plo && p0 + 8 <= phi;
+        if (whole && quads) {
+            const double2 *x = reinterpret_cast<const double2 *>(X + (long long)r * ld + p0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { const double2 t = x[q]; v[2 * q] = t.x; v[2 * q + 1] = t.y; }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int p = p0 + q;
+                const bool in = whole || (live && p >= plo && p < phi);
+                v[q] = in ? (o.trans ? X[(long long)p * ld + r] : X[(long long)r * ld + p]) : 0.0;
+            }
         }
-    } else {       // memory rows are r: a warp reads 32 consecutive p of one r
-        for (int it = 0; it < 8; ++it) {
-            const int rl = it * 4 + (tid >> 6), pl = tid & 63;
-            T[rl][pl] = oz_load(X, ld, 0, rows, k, tri, ks, r0 + rl, p0 + pl);
+        if (o.ks) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (p0 + q < k) v[q] *= o.ks[p0 + q];
+        }
+    };
+    int mx = INT_MIN / 2;
+    for (int kb = kb_lo + warp; kb < kb_hi; kb += 8) {
+        double v[8];
+        load(kb, v);
+        int h = 0;                                     // largest high word of a magnitude: orders them by exponent
+#pragma unroll
+        for (int q = 0; q < 8; ++q) h = max(h, __double2hiint(v[q]) & 0x7FFFFFFF);
+        if (h >= 0x00100000) {
+            mx = max(mx, (h >> 20) - 1022);
+        } else {                                       // zeros and subnormal numbers only
+#pragma unroll
+            for (int q = 0; q < 8; ++q) mx = max(mx, oz_frexp_exp(v[q]));
         }
     }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o.trans ? 16 : 1));
+    if (half == 0) top[warp][rl] = mx;
     __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31;
-    const int rl = (warp & 1) * 16 + (lane >> 1);          // row within the tile
-    const int kb = warp >> 1;                              // k block within the tile (0..3)
-    const int half = lane & 1;                             // columns 8 half .. 8 half + 7 of the k block
-    const int r = r0 + rl, pb = p0 + kb * 16 + half * 8;
-    if (r >= rows_pad || pb >= k_pad) return;
-    const int ex = (r < rows) ? e[z * rows_pad + r] : -4000;
-    long long f[8];
+    int ex = top[0][rl];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) f[q] = (ex > -2000) ? oz_fixed56(T[rl][kb * 16 + half * 8 + q], ex) : 0;
-    const int kblocks = k_pad / 16, tiles = rows_pad / tile_rows;
-    const int rr = r % tile_rows;
-    const long long oblk = ((long long)z * tiles + r / tile_rows) * kblocks + (pb >> 4);
-    __nv_bfloat16 *dst = out + oblk * (OZ_S * tile_rows * 16) + rr * 16 + ((half ^ (rr >> 2)) & 1) * 8;
-    const int sstride = tile_rows * 16;
-    uint32_t w[OZ_S][4];
+    for (int w = 1; w < 8; ++w) ex = max(ex, top[w][rl]);
+    if (warp == 0 && half == 0) o.e[(long long)z * o.rows_pad + r] = ex;
+    if (!live || ex <= -2000) ex = -4000;
+    // row tiles read the k range of their own triangle rounded out to their height: blocks
+    // within 256 rows of it are written as zeros, those beyond are never read
+    const int w_lo = o.tri == TRI_UPPER ? max(0, min(kblocks, r0 / 16) - 16) : 0;
+    const int w_hi = o.tri == TRI_LOWER ? min(kblocks, r0 / 16 + 17) : kblocks;
+    __nv_bfloat16 *tile = o.out + ((long long)z * (o.rows_pad / o.tile_rows) + r / o.tile_rows) * kblocks * (OZ_S * o.tile_rows * 16) +
+                          (r % o.tile_rows) * 16 + ((half ^ (r >> 2)) & 1) * 8;
+    for (int kb = w_lo + warp; kb < w_hi; kb += 8) {
+        double v[8];
+        long long f[8];
+        uint32_t w[OZ_S][4];
+        load(kb, v);
 #pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-        uint32_t ba[OZ_S], bb[OZ_S];
-        oz_digits(f[q], ba);
-        oz_digits(f[q + 1], bb);
+        for (int q = 0; q < 8; ++q) f[q] = (ex > -2000) ? oz_fixed56(v[q], ex) : 0;
 #pragma unroll
-        for (int t = 0; t < OZ_S; ++t) w[t][q >> 1] = __byte_perm(ba[t], bb[t], 0x7632);   // two upper halves
+        for (int q = 0; q < 8; q += 2) {
+            uint32_t ba[OZ_S], bb[OZ_S];
+            oz_digits(f[q], ba);
+            oz_digits(f[q + 1], bb);
+#pragma unroll
+            for (int t = 0; t < OZ_S; ++t) w[t][q >> 1] = __byte_perm(ba[t], bb[t], 0x7632);   // two upper halves
+        }
+        __nv_bfloat16 *dst = tile + (long long)kb * (OZ_S * o.tile_rows * 16);
+#pragma unroll
+        for (int t = 0; t < OZ_S; ++t)
+            *reinterpret_cast<uint4 *>(dst + t * o.tile_rows * 16) = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
     }
-#pragma unroll
-    for (int t = 0; t < OZ_S; ++t)
-        *reinterpret_cast<uint4 *>(dst + t * sstride) = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
-}
-
-__global__ void fill_int_kernel(int *x, long long n, int v)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        x[i] = v;
 }
 
 }  // namespace
 
-size_t oz_gemm_workspace_bytes(const GemmArgs &g)
-{
-    const long long kp = (g.k + 15) / 16 * 16;
-    const long long mp = (g.m + OZ_BM - 1) / OZ_BM * OZ_BM, np = (g.n + OZ_BN - 1) / OZ_BN * OZ_BN;
-    return (size_t)(OZ_S * (mp + np) * kp * g.batch) * 2 + (size_t)(mp + np) * g.batch * sizeof(int) + 2048;
-}
-
 namespace {
 struct OzLayout {
-    int kp, mp, np;
+    int kp, mp, np;                        // k, rows of A, rows of B padded
     __nv_bfloat16 *sa, *sb;
     int *ea, *eb;
 };
@@ -583,25 +559,24 @@ OzLayout oz_layout(const GemmArgs &g, void *ws)
 }
 }  // namespace
 
-// operand preparation: exponents and pre-tiled slices of op(A) and op(B) into ws
+size_t oz_gemm_workspace_bytes(const GemmArgs &g)
+{
+    const long long kp = (g.k + 15) / 16 * 16;
+    const long long mp = (g.m + OZ_BM - 1) / OZ_BM * OZ_BM, np = (g.n + OZ_BN - 1) / OZ_BN * OZ_BN;
+    return (size_t)(OZ_S * (mp + np) * kp * g.batch) * 2 + (size_t)(mp + np) * g.batch * sizeof(int) + 2048;
+}
+
+// operand preparation: exponents and slices of op(A) and op(B) into ws
 int oz_gemm_prepare(const GemmArgs &g, void *ws, cudaStream_t s)
 {
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return 0;
     const OzLayout L = oz_layout(g, ws);
     const int triB = g.triB == TRI_LOWER ? TRI_UPPER : (g.triB == TRI_UPPER ? TRI_LOWER : TRI_NONE);
-    fill_int_kernel<<<64, 256, 0, s>>>(L.ea, (long long)(L.mp + L.np) * g.batch, INT_MIN / 2); count_launch();
     // op(A) rows are memory rows unless A is transposed; op(B) columns are memory rows when B is transposed
     OzOperand oa{(const double *)g.A, g.lda, g.sA, g.ta, g.m, g.triA, (const double *)g.kscale, L.mp, OZ_BM, L.ea, L.sa};
     OzOperand ob{(const double *)g.B, g.ldb, g.sB, g.tb ? 0 : 1, g.n, triB, nullptr, L.np, OZ_BN, L.eb, L.sb};
-    {
-        const int nA = oz_exp_blocks(oa, g.k), nB = oz_exp_blocks(ob, g.k);
-        oz_exp_kernel<<<dim3(nA + nB, 1, g.batch), 256, 0, s>>>(oa, ob, g.k, nA); count_launch();
-    }
-    {
-        const int pt = (L.kp + 63) / 64;
-        const int nA = pt * (L.mp / 32), nB = pt * (L.np / 32);
-        oz_slice_kernel<<<dim3(nA + nB, 1, g.batch), 256, 0, s>>>(oa, ob, g.k, L.kp, nA); count_launch();
-    }
+    const int nA = L.mp / 16, nB = L.np / 16;
+    oz_prepare_kernel<<<dim3(nA + nB, 1, g.batch), 256, 0, s>>>(oa, ob, g.k, L.kp, nA); count_launch();
     return 0;
 }
 
@@ -609,7 +584,6 @@ int oz_gemm_prepare(const GemmArgs &g, void *ws, cudaStream_t s)
 int oz_gemm_run(const GemmArgs &g, void *ws, int *err, cudaStream_t s)
 {
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return 0;
-    if (!ensure_dynamic_smem((const void *)oz_gemm_kernel, OZ_SMEM_BYTES)) return -2;
     const OzLayout L = oz_layout(g, ws);
     OzArgs a;
     a.sa = L.sa; a.sb = L.sb; a.kblocks = L.kp / 16;
@@ -627,17 +601,19 @@ int oz_gemm_run(const GemmArgs &g, void *ws, int *err, cudaStream_t s)
         a.alpha_e = a.alpha_e_valid ? ex - 1 : 0;
         a.alpha_neg = (a.alpha_e_valid && g.alpha < 0) ? 1 : 0;
     }
-    dim3 grid(((g.n + OZ_BN - 1) / OZ_BN) * ((g.m + OZ_BM - 1) / OZ_BM), 1, g.batch);
-    oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM_BYTES, s>>>(a); count_launch();
+    const int tiles = ((g.n + OZ_BN - 1) / OZ_BN) * ((g.m + OZ_BM - 1) / OZ_BM);
+    if (!ensure_dynamic_smem((const void *)oz_gemm_kernel, OZ_SMEM_BYTES)) return -2;
+    oz_gemm_kernel<<<dim3(tiles, 1, g.batch), OZ_THREADS, OZ_SMEM_BYTES, s>>>(a);
+    count_launch();
     return 0;
 }
 
-// estimate of the slice engine's time in microseconds: the four launches, prologue and
-// epilogue, then the k blocks of the tiles a busiest SM takes in turn
+// estimate of the slice engine's time in microseconds: the two launches, prologue and epilogue,
+// then 1 us for each k block of the tiles a busiest SM takes in turn (preparation included)
 double oz_gemm_time_us(const GemmArgs &g)
 {
     const double mt = (g.m + OZ_BM - 1) / OZ_BM, nt = (g.n + OZ_BN - 1) / OZ_BN;
-    return 30.0 + std::ceil((g.lowerC ? 0.5 : 1.0) * mt * nt * g.batch / 152.0) * (g.k / OZ_BK) * 0.56;
+    return 11.0 + std::ceil((g.lowerC ? 0.5 : 1.0) * mt * nt * g.batch / 152.0) * (g.k / OZ_BK);
 }
 
 int oz_gemm_launch(const GemmArgs &g, void *ws, int *err, cudaStream_t s)

@@ -274,9 +274,9 @@ void gemm(pssd_handle h, const GemmArgs &g0)
     double fl = h->prof ? 2.0 * gemm_macs(g) : 0.0;
     Mark mk = mark(h);
     if (g.mode == GM_OZ && !h->derr) g.mode = GM_DF;   // (no error flag outside a guarded call)
-    // Small products: the slice engine's four launches and its tile latency dominate, and the
-    // FP64 pipes finish first (64^3: 5 us against 28 us; 256^3: 38 us against 44 us; 384^3: 115 us
-    // against 50 us, so the estimates decide).  Upstream of the mixed mode's FP32 iteration the
+    // Small products: the slice engine's two launches and its tile latency dominate, and the
+    // FP64 pipes finish first (64^3: 3 us against 14 us; 192^3: 16 against 24; 256^3: 35 against
+    // 27; the estimates decide).  Upstream of the mixed mode's FP32 iteration the
     // engines are pinned -- float pairs for thin or tiny products, slices for the rest: the
     // iteration turns a flipped last bit of its input into a change of the size of its own
     // error, so mixed results would otherwise move with every choice made here.
@@ -312,8 +312,8 @@ void gemm(pssd_handle h, const GemmArgs &g0)
     const double opA = (double)g.batch * g.m * g.k, opB = (double)g.batch * g.n * g.k;
     if (g.mode == GM_OZ) {
         void *ws = walloc(h, oz_gemm_workspace_bytes(g));
-        {   // exponent pass (8 B read) + slicing pass (8 B read, 8 slices x 2 B written) per element
-            Timed t(h, K_OZPREP, 0, 32.0 * (opA + opB));
+        {   // 8 B read and eight slices of 2 B written per element
+            Timed t(h, K_OZPREP, 0, 24.0 * (opA + opB));
             oz_gemm_prepare(g, ws, h->stream);
         }
         Timed t(h, K_OZGEMM, fl);
