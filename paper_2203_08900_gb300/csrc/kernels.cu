@@ -14,8 +14,6 @@
 #include "mbar.cuh"
 #include "pssd_internal.h"
 
-#include <cooperative_groups.h>
-
 #include <math.h>
 
 #include <type_traits>
@@ -1787,205 +1785,188 @@ void dot_vec(const double *x, const double *y, int n, double *out, cudaStream_t 
 // Krylov loops in one launch.  Step by step, a Lanczos step takes four launches
 // (product, alpha, three-term update, beta with the new vector) and a power
 // step three or four; the recursion's nodes, the bounds of small inputs and
-// the shift screening run such loops hundreds of times on operators whose
-// matrix sits in L2.  Here one cluster of KRY_CLUSTER CTAs runs a whole loop.
-// CTA c owns rows [c R, (c + 1) R) of the operator, R = ceil(m / KRY_CLUSTER);
-// every CTA keeps the whole current and previous vectors in shared memory.  A
-// dot product is summed per CTA (warps, then warps in order), then across the
-// cluster through distributed shared memory in rank order, so every CTA holds
-// the same scalar to the bit.  A new vector is all-gathered by each CTA storing
-// its rows into every CTA's buffer.  Each exchange ends at a cluster barrier, a
-// hardware barrier that every thread of every CTA reaches equally often (all
-// loop bounds are uniform across the cluster): no thread waits on a flag.
+// the shift screening run such loops hundreds of times on operators of order
+// at most KRY_MAX_M.  What bounds a loop is the FP64 pipe (m^2 multiply-adds a
+// step, 2 per clock and SM) and then the exchanges, so the rows are spread over
+// m / 8 CTAs of 8 warps, one row (and, for L^T, one column) to a warp, held in
+// its registers for the whole loop.  A product's entries go through global
+// memory to every CTA (two buffers in turn) behind one grid barrier; the dot
+// products, the three-term update and the normalisation are then done by every
+// CTA for itself, in the same order, so all hold the same bits.  The launch is
+// cooperative -- all CTAs are resident before any waits -- and a wait that runs
+// out of polls makes the loop return NaN.
+// Sums: 32 consecutive entries by a shuffle tree, the trees' results in order,
+// over KRY_SEGMENTS equal segments of the vector first, then those in order.
+// Measured, 24 Lanczos steps: m = 128 KRYA, m = 1000 KRYB; on one cluster of 8
+// CTAs, which these loops ran on before, 440 and 1940 us.
 // ---------------------------------------------------------------------------
-constexpr int KRY_CLUSTER = 8, KRY_THREADS = 1024, KRY_WARPS = KRY_THREADS / 32;
-constexpr int KRY_ROWS = KRY_MAX_M / KRY_CLUSTER;      // rows (and columns) owned by a CTA, at most
-constexpr int KRY_GROUPS = KRY_THREADS / KRY_ROWS;     // row groups of the transposed product
-constexpr int KRY_SMEM = (4 * KRY_MAX_M + KRY_ROWS + KRY_GROUPS * KRY_ROWS) * (int)sizeof(double);
-static_assert(KRY_THREADS % KRY_ROWS == 0 && KRY_SMEM <= 48 * 1024, "Krylov kernel layout");
+constexpr int KRY_ROWS = 8, KRY_THREADS = 32 * KRY_ROWS, KRY_SEGMENTS = 8;
+constexpr int KRY_T = KRY_MAX_M / 32;                  // entries of a row per lane
+constexpr int KRY_GROUPS = KRY_SEGMENTS * (KRY_MAX_M / KRY_SEGMENTS / 32);   // sums of 32 entries, at most
+constexpr unsigned int KRY_WAIT_LIMIT = 1u << 22;
 
-namespace cg = cooperative_groups;
-
-// sum of x over the CTA, returned to every thread
-__device__ double kry_block_sum(double x, double *red, double *bc)
+// every CTA of the grid has arrived (count: 0 at launch; target: arrivals so far times CTAs)
+__device__ __forceinline__ bool kry_grid_sync(unsigned int *count, unsigned int target, int *sm_ok)
 {
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < KRY_WARPS; ++w) s += red[w];
-        *bc = s;
+        unsigned int v;
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        int ok = 0;
+        for (unsigned int it = 0; it < KRY_WAIT_LIMIT; ++it) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            if (v >= target) { ok = 1; break; }
+        }
+        *sm_ok = ok;
     }
     __syncthreads();
-    return *bc;
+    return *sm_ok != 0;
 }
 
-// sum over the cluster of the CTAs' partial sums `part`, returned to every thread of
-// every CTA.  Two slots alternate: a slot is rewritten only after another cluster
-// barrier, by which time every CTA has read it.
-__device__ double kry_cluster_sum(cg::cluster_group &cl, double part, double *slot, int &turn, double *bc)
-{
-    double *my = slot + turn;
-    turn ^= 1;
-    if (threadIdx.x == 0) *my = part;
-    cl.sync();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int c = 0; c < KRY_CLUSTER; ++c) s += *cl.map_shared_rank(my, c);
-        *bc = s;
-    }
-    __syncthreads();
-    return *bc;
-}
-
-// rows r0 .. r0 + nr - 1 of A x (tri: of L x, L lower triangular) -> wl; one warp per row
-__device__ void kry_rows(const double *__restrict__ A, long long lda, bool tri, const double *x, double *wl,
-                         int r0, int nr, int m)
+// sum of f(i), i < m, returned to every thread: groups of 32 from the start of each segment of
+// `seg` entries, the groups of a segment in order, the segments in order
+template <class F>
+__device__ __forceinline__ double kry_sum(int m, int seg, F f, double *red, double *bc)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = warp; i < nr; i += KRY_WARPS) {
-        const double *row = A + (long long)(r0 + i) * lda;
-        const int len = tri ? r0 + i + 1 : m;
-        double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        int k = lane;
-        for (; k + 224 < len; k += 256) {   // eight independent loads in flight per lane
-            double r[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) r[q] = __ldg(row + k + 32 * q);
-#pragma unroll
-            for (int q = 0; q < 8; ++q) a[q] = fma(r[q], x[k + 32 * q], a[q]);
-        }
-        if (k + 96 < len) {
-            double r[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) r[q] = __ldg(row + k + 32 * q);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] = fma(r[q], x[k + 32 * q], a[q]);
-            k += 128;
-        }
-        for (; k < len; k += 32) a[0] = fma(__ldg(row + k), x[k], a[0]);
-        double s = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) wl[i] = s;
+    const int per = (seg + 31) / 32, ns = (m + seg - 1) / seg;
+    for (int g = warp; g < ns * per; g += KRY_ROWS) {
+        const int s0 = (g / per) * seg, i = s0 + (g % per) * 32 + lane;
+        double x = (i < m && i < s0 + seg) ? f(i) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        if (lane == 0) red[g] = x;
     }
     __syncthreads();
-}
-
-// entries r0 .. r0 + nr - 1 of L^T u (L lower triangular) -> wl: thread (g, c) sums
-// L[p][r0 + c] u[p] over p = r0 + g, r0 + g + KRY_GROUPS, ... (a warp reads 32
-// consecutive entries of a row), then the groups' sums are added in order
-__device__ void kry_tri_t_cols(const double *__restrict__ A, long long lda, const double *u, double *wl,
-                               double *colp, int r0, int nr, int m)
-{
-    const int c = threadIdx.x % KRY_ROWS, g = threadIdx.x / KRY_ROWS;
-    double acc = 0.0;
-    if (c < nr) {
-        const int col = r0 + c;
-        for (int p = max(r0 + g, col - (col - r0 - g) % KRY_GROUPS); p < m; p += KRY_GROUPS)
-            if (p >= col) acc = fma(__ldg(A + (long long)p * lda + col), u[p], acc);
-    }
-    colp[g * KRY_ROWS + c] = acc;
-    __syncthreads();
-    for (int i = threadIdx.x; i < nr; i += KRY_THREADS) {
+    if (warp == 0) {
+        double p = 0.0;                                // lane c: segment c
+        if (lane < ns)
+            for (int j = 0; j < per; ++j) p += red[lane * per + j];
         double s = 0.0;
-        for (int q = 0; q < KRY_GROUPS; ++q) s += colp[q * KRY_ROWS + i];
-        wl[i] = s;
+        for (int c = 0; c < ns; ++c) s += __shfl_sync(0xffffffffu, p, c);
+        if (lane == 0) *bc = s;
     }
     __syncthreads();
+    return *bc;
 }
 
-// scale * src[0 .. nr) -> dst[r0 .. r0 + nr) in every CTA of the cluster, then a cluster barrier
-__device__ void kry_gather(cg::cluster_group &cl, const double *src, double scale, double *dst, int r0, int nr)
+// row . x for a row of `len` entries held by a warp (lane l: entries l, l + 32, ...; zero
+// beyond): eight running sums over blocks of 256, a block of 128 into four of them where one is
+// left, the rest into the first, added pairwise and over the lanes by a shuffle tree
+__device__ __forceinline__ double kry_row_dot(const double *row, int len, const double *x, int lane)
 {
-    for (int c = 0; c < KRY_CLUSTER; ++c) {
-        double *rd = cl.map_shared_rank(dst, c);
-        for (int i = threadIdx.x; i < nr; i += KRY_THREADS) rd[r0 + i] = src[i] * scale;
+    double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const int nb = max(0, (len - 224 - lane + 255) / 256);         // whole blocks of this lane (len - 224 - lane > 256 b)
+    const bool four = lane + 256 * nb + 96 < len;
+    const int nb_all = max(0, (len - 224 - 31 + 255) / 256);       // of every lane
+#pragma unroll
+    for (int t = 0; t < KRY_T; ++t) {
+        if (32 * t >= len) break;
+        const int b = t >> 3, q = t & 7, i = lane + 32 * t;
+        const double v = row[t];
+        if (b < nb_all || q == 0) {
+            if (i < len) a[q] = fma(v, x[i], a[q]);
+        } else {
+            const bool own = b < nb || (b == nb && four && q < 4);
+            if (i < len) {
+                if (own) a[q] = fma(v, x[i], a[q]);
+                else a[0] = fma(v, x[i], a[0]);
+            }
+        }
     }
-    cl.sync();
+    double s = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    return s;
 }
 
 template <int OP>
-__global__ void __cluster_dims__(KRY_CLUSTER, 1, 1) __launch_bounds__(KRY_THREADS, 1)
-krylov_cluster_kernel(const double *__restrict__ A, long long lda, int m, int steps, int power, uint64_t seed,
-                      double *out)
+__global__ void __launch_bounds__(KRY_THREADS, 1)
+krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps, int power, uint64_t seed, double *out,
+                   double *ex, unsigned int *count)
 {
-    extern __shared__ __align__(16) double kry_sm[];
-    __shared__ double red[KRY_WARPS], slot[2], bc;
-    cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank();
-    const int R = (m + KRY_CLUSTER - 1) / KRY_CLUSTER;
-    const int r0 = min(m, rank * R), nr = min(m, r0 + R) - r0;
-    double *cur = kry_sm, *prv = cur + KRY_MAX_M, *nxt = prv + KRY_MAX_M, *ub = nxt + KRY_MAX_M;
-    double *wl = ub + KRY_MAX_M, *colp = wl + KRY_ROWS;
+    __shared__ double cur[KRY_MAX_M], prv[KRY_MAX_M], w[KRY_MAX_M];
+    __shared__ double red[KRY_GROUPS + 8], bc;
+    __shared__ int sm_ok;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r = blockIdx.x * KRY_ROWS + warp;
+    const int seg = (m + KRY_SEGMENTS - 1) / KRY_SEGMENTS;
+    unsigned int arrived = 0;
     int turn = 0;
-    // the starting vector, whole in every CTA (same entries, same summation order)
-    double sq = 0.0;
-    for (int i = threadIdx.x; i < m; i += KRY_THREADS) {
-        const double g = gauss_at(seed, (uint64_t)i);
-        cur[i] = g;
-        prv[i] = 0.0;
-        sq += g * g;
+    bool ok = true;
+    // entry r of a vector (lane 0's v) -> dst, whole in every CTA
+    auto exchange = [&](double v, double *dst) {
+        double *buf = ex + turn * m;
+        turn ^= 1;
+        if (r < m && lane == 0) __stcg(buf + r, v);
+        arrived += gridDim.x;
+        if (ok) ok = kry_grid_sync(count, arrived, &sm_ok);
+        for (int i = tid; i < m; i += KRY_THREADS) dst[i] = __ldcg(buf + i);
+        __syncthreads();
+    };
+    // this warp's row of A (of L), and column of L
+    const int rlen = r < m ? (OP == KRY_SYM ? m : r + 1) : 0;
+    double row[KRY_T], col[OP == KRY_TRI_PAIR ? KRY_T : 1];
+#pragma unroll
+    for (int t = 0; t < KRY_T; ++t) {
+        const int i = lane + 32 * t;
+        row[t] = i < rlen ? __ldg(A + (long long)r * lda + i) : 0.0;
+        if (OP == KRY_TRI_PAIR) col[t] = (r < m && i >= r && i < m) ? __ldg(A + (long long)i * lda + r) : 0.0;
     }
-    sq = kry_block_sum(sq, red, &bc);
+    exchange(r < m && lane == 0 ? gauss_at(seed, (uint64_t)r) : 0.0, cur);
+    const double sq = kry_sum(m, KRY_MAX_M, [&](int i) { return cur[i] * cur[i]; }, red, &bc);
     const double inv0 = sq > 0.0 ? 1.0 / sqrt(sq) : 0.0;
-    for (int i = threadIdx.x; i < m; i += KRY_THREADS) cur[i] *= inv0;
-    cl.sync();   // every CTA has started (its shared memory exists) before the first remote access
-    auto apply = [&](const double *x) {   // the CTA's rows of op(A) x -> wl
+    for (int i = tid; i < m; i += KRY_THREADS) { cur[i] *= inv0; prv[i] = 0.0; }
+    __syncthreads();
+    auto apply = [&]() {                               // op(A) cur -> w
         if (OP == KRY_SYM) {
-            kry_rows(A, lda, false, x, wl, r0, nr, m);
+            exchange(kry_row_dot(row, rlen, cur, lane), w);
         } else {
-            kry_rows(A, lda, true, x, wl, r0, nr, m);         // u = L x, own rows
-            kry_gather(cl, wl, 1.0, ub, r0, nr);               // u whole in every CTA
-            kry_tri_t_cols(A, lda, ub, wl, colp, r0, nr, m);   // L^T u, own entries
+            exchange(kry_row_dot(row, rlen, cur, lane), w);                    // u = L x
+            exchange(kry_row_dot(col, r < m ? m : 0, w, lane), w);             // L^T u (zeros above the diagonal)
         }
     };
     if (power == 0) {
         double beta_prev = 0.0;
         for (int j = 0; j < steps; ++j) {
-            apply(cur);
-            double pa = 0.0;
-            for (int i = threadIdx.x; i < nr; i += KRY_THREADS) pa += cur[r0 + i] * wl[i];
-            const double alpha = kry_cluster_sum(cl, kry_block_sum(pa, red, &bc), slot, turn, &bc);
-            double pb = 0.0;
-            for (int i = threadIdx.x; i < nr; i += KRY_THREADS) {
-                const double w = wl[i] - alpha * cur[r0 + i] - beta_prev * prv[r0 + i];
-                wl[i] = w;
-                pb += w * w;
-            }
-            const double beta = sqrt(kry_cluster_sum(cl, kry_block_sum(pb, red, &bc), slot, turn, &bc));
-            if (rank == 0 && threadIdx.x == 0) { out[j] = alpha; out[steps + 1 + j] = beta; }
-            kry_gather(cl, wl, beta > 0.0 ? 1.0 / beta : 0.0, nxt, r0, nr);
-            double *t = prv; prv = cur; cur = nxt; nxt = t;
+            apply();
+            const double alpha = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, &bc);
+            for (int i = tid; i < m; i += KRY_THREADS) w[i] = w[i] - alpha * cur[i] - beta_prev * prv[i];
+            __syncthreads();
+            const double beta = sqrt(kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, &bc));
+            if (blockIdx.x == 0 && tid == 0) { out[j] = ok ? alpha : NAN; out[steps + 1 + j] = ok ? beta : NAN; }
+            const double scale = beta > 0.0 ? 1.0 / beta : 0.0;
+            for (int i = tid; i < m; i += KRY_THREADS) { prv[i] = cur[i]; cur[i] = w[i] * scale; }
+            __syncthreads();
             beta_prev = beta;
         }
     } else {
         for (int it = 0; it < power; ++it) {
-            apply(cur);
-            double pb = 0.0;
-            for (int i = threadIdx.x; i < nr; i += KRY_THREADS) pb += wl[i] * wl[i];
-            const double nrm = sqrt(kry_cluster_sum(cl, kry_block_sum(pb, red, &bc), slot, turn, &bc));
-            kry_gather(cl, wl, nrm > 0.0 ? 1.0 / nrm : 0.0, nxt, r0, nr);
-            double *t = cur; cur = nxt; nxt = t;
+            apply();
+            const double nrm = sqrt(kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, &bc));
+            const double scale = nrm > 0.0 ? 1.0 / nrm : 0.0;
+            for (int i = tid; i < m; i += KRY_THREADS) cur[i] = w[i] * scale;
+            __syncthreads();
         }
-        apply(cur);
-        double pa = 0.0;
-        for (int i = threadIdx.x; i < nr; i += KRY_THREADS) pa += cur[r0 + i] * wl[i];
-        const double rq = kry_cluster_sum(cl, kry_block_sum(pa, red, &bc), slot, turn, &bc);
-        if (rank == 0 && threadIdx.x == 0) out[0] = rq;
+        apply();
+        const double rq = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, &bc);
+        if (blockIdx.x == 0 && tid == 0) out[0] = ok ? rq : NAN;
     }
-    cl.sync();   // no CTA leaves while another may still read its shared memory
 }
 
-bool krylov_cluster(const double *A, long long lda, int op, int m, int steps, int power, uint64_t seed, double *out,
-                    cudaStream_t s)
+size_t krylov_scratch_doubles(int m) { return 2 * (size_t)m + 8; }
+
+bool krylov_fused(const double *A, long long lda, int op, int m, int steps, int power, uint64_t seed, double *out,
+                  double *scratch, cudaStream_t s)
 {
     if (m < 1 || m > KRY_MAX_M || steps < 0 || power < 0) return false;
-    if (op == KRY_SYM)
-        krylov_cluster_kernel<KRY_SYM><<<KRY_CLUSTER, KRY_THREADS, KRY_SMEM, s>>>(A, lda, m, steps, power, seed, out);
-    else
-        krylov_cluster_kernel<KRY_TRI_PAIR><<<KRY_CLUSTER, KRY_THREADS, KRY_SMEM, s>>>(A, lda, m, steps, power, seed,
-                                                                                      out);
+    unsigned int *count = (unsigned int *)(scratch + 2 * (size_t)m);
+    if (cudaMemsetAsync(count, 0, sizeof(unsigned int), s) != cudaSuccess) return false;
+    void *args[] = {&A, &lda, &m, &steps, &power, &seed, &out, &scratch, &count};
+    const void *kernel = op == KRY_SYM ? (const void *)krylov_grid_kernel<KRY_SYM>
+                                       : (const void *)krylov_grid_kernel<KRY_TRI_PAIR>;
+    if (cudaLaunchCooperativeKernel(kernel, dim3((m + KRY_ROWS - 1) / KRY_ROWS), dim3(KRY_THREADS), args, 0, s) !=
+        cudaSuccess)
+        return false;
     count_launch();
     return true;
 }

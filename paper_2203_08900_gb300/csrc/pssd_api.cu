@@ -922,14 +922,24 @@ int ns_refine(pssd_handle h, double *Y, int m, double tol, int max_it, double *r
     return PSSD_OK;
 }
 
-// The operator of a Krylov loop in the form the one-launch cluster kernel takes
-// (krylov_cluster: y = A x, or y = L^T (L x) for lower triangular L); A = null: none,
+// The operator of a Krylov loop in the form the one-launch kernel takes
+// (krylov_fused: y = A x, or y = L^T (L x) for lower triangular L); A = null: none,
 // the loop then runs step by step through its `apply` callback.
 struct KryFused {
     const double *A = nullptr;
     long long lda = 0;
     int op = KRY_SYM;
     bool usable(int m) const { return A && m >= 1 && m <= KRY_MAX_M; }
+    void run(pssd_handle h, int m, int steps, int power, uint64_t seed, double *out) const
+    {
+        Mark mk = mark(h);
+        double *scratch = dalloc(h, krylov_scratch_doubles(m));
+        if (!krylov_fused(A, lda, op, m, steps, power, seed, out, scratch, h->stream)) {
+            h->last_err = std::string("Krylov launch: ") + cudaGetErrorString(cudaGetLastError());
+            throw Fail{PSSD_ERR_CUDA};
+        }
+        release(h, mk);
+    }
 };
 
 // power iteration estimate of lambda_max of an SPD operator given by `apply` (or by `kf`:
@@ -940,7 +950,7 @@ void power_device(pssd_handle h, int n, F apply, double *v, double *w, double *d
 {
     if (kf && kf->usable(n) && iters > 0) {
         Timed t(h, K_GEMV, (iters + 1) * 2.0 * n * (double)n, (iters + 1) * 8.0 * n * (double)n);
-        krylov_cluster(kf->A, kf->lda, kf->op, n, 0, iters, 0x5eedull, dscal, h->stream);
+        kf->run(h, n, 0, iters, 0x5eedull, dscal);
     } else {
         {
             Timed t(h, K_HBM, 0, 24.0 * n);
@@ -1241,7 +1251,7 @@ void lanczos_device(pssd_handle h, int m, F apply, uint64_t seed, int steps, dou
 {
     if (kf && kf->usable(m)) {
         Timed t(h, K_GEMV, steps * 2.0 * m * (double)m, steps * 8.0 * m * (double)m);
-        krylov_cluster(kf->A, kf->lda, kf->op, m, steps, 0, seed, ab, h->stream);
+        kf->run(h, m, steps, 0, seed, ab);
         return;
     }
     Mark mk = mark(h);

@@ -168,18 +168,20 @@ void dot_vec(const double *x, const double *y, int n, double *out, cudaStream_t 
 void lanczos_update(double *w, const double *v, const double *vprev, const double *alpha, const double *beta, int n,
                     cudaStream_t s);
 
-// Krylov loops in one launch for operators of order m <= KRY_MAX_M (one thread-block
-// cluster; see kernels.cu).  Operators: KRY_SYM y = A x (A symmetric, full storage);
+// Krylov loops in one cooperative launch for operators of order m <= KRY_MAX_M (see
+// kernels.cu).  Operators: KRY_SYM y = A x (A symmetric, full storage);
 // KRY_TRI_PAIR y = L^T (L x) (L lower triangular, entries above the diagonal not read).
 // The starting vector is the Gaussian vector fill_gaussian(v, m, 1, m, seed) makes.
 //   power == 0: `steps` Lanczos steps; out[j] = alpha_j (j < steps) and
 //               out[steps + 1 + j] = beta_j, the layout of the step-by-step loop.
 //   power  > 0: `power` normalised power steps, then out[0] = v^T A v.
-// Returns false (nothing launched) if m is outside [1, KRY_MAX_M].
+// scratch: krylov_scratch_doubles(m) doubles.  Returns false (nothing launched) if m is outside
+// [1, KRY_MAX_M] or the launch failed.
 constexpr int KRY_MAX_M = 1024;
 enum KryOp { KRY_SYM = 0, KRY_TRI_PAIR = 1 };
-bool krylov_cluster(const double *A, long long lda, int op, int m, int steps, int power, uint64_t seed, double *out,
-                    cudaStream_t s);
+size_t krylov_scratch_doubles(int m);
+bool krylov_fused(const double *A, long long lda, int op, int m, int steps, int power, uint64_t seed, double *out,
+                  double *scratch, cudaStream_t s);
 void scale_columns(double *X, long long ldx, int m, int n, const double *d, int use_sqrt_abs,
                    cudaStream_t s);
 void sign_fix_columns(double *X, long long ldx, int m, int n, cudaStream_t s);
