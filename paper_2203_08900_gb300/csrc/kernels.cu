@@ -1797,7 +1797,7 @@ void dot_vec(const double *x, const double *y, int n, double *out, cudaStream_t 
 // out of polls makes the loop return NaN.
 // Sums: 32 consecutive entries by a shuffle tree, the trees' results in order,
 // over KRY_SEGMENTS equal segments of the vector first, then those in order.
-// Measured, 24 Lanczos steps: m = 128 KRYA, m = 1000 KRYB; on one cluster of 8
+// Measured, 24 Lanczos steps: m = 128 190 us, m = 1000 400 us; on one cluster of 8
 // CTAs, which these loops ran on before, 440 and 1940 us.
 // ---------------------------------------------------------------------------
 constexpr int KRY_ROWS = 8, KRY_THREADS = 32 * KRY_ROWS, KRY_SEGMENTS = 8;
@@ -1825,9 +1825,11 @@ __device__ __forceinline__ bool kry_grid_sync(unsigned int *count, unsigned int 
 }
 
 // sum of f(i), i < m, returned to every thread: groups of 32 from the start of each segment of
-// `seg` entries, the groups of a segment in order, the segments in order
+// `seg` entries, the groups of a segment in order, the segments in order.  root: the square root
+// of the sum instead, and its reciprocal (0 for 0) in bc[1], by one warp (each takes some ten
+// dependent FP64 instructions, which eight warps would issue one after the other)
 template <class F>
-__device__ __forceinline__ double kry_sum(int m, int seg, F f, double *red, double *bc)
+__device__ __forceinline__ double kry_sum(int m, int seg, F f, double *red, double *bc, bool root = false)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int per = (seg + 31) / 32, ns = (m + seg - 1) / seg;
@@ -1844,10 +1846,15 @@ __device__ __forceinline__ double kry_sum(int m, int seg, F f, double *red, doub
             for (int j = 0; j < per; ++j) p += red[lane * per + j];
         double s = 0.0;
         for (int c = 0; c < ns; ++c) s += __shfl_sync(0xffffffffu, p, c);
-        if (lane == 0) *bc = s;
+        if (root) {
+            s = sqrt(s);
+            const double inv = s > 0.0 ? 1.0 / s : 0.0;
+            if (lane == 0) bc[1] = inv;
+        }
+        if (lane == 0) bc[0] = s;
     }
     __syncthreads();
-    return *bc;
+    return bc[0];
 }
 
 // row . x for a row of `len` entries held by a warp (lane l: entries l, l + 32, ...; zero
@@ -1885,7 +1892,7 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
                    double *ex, unsigned int *count)
 {
     __shared__ double cur[KRY_MAX_M], prv[KRY_MAX_M], w[KRY_MAX_M];
-    __shared__ double red[KRY_GROUPS + 8], bc;
+    __shared__ double red[KRY_GROUPS + 8], bc[2];
     __shared__ int sm_ok;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int r = blockIdx.x * KRY_ROWS + warp;
@@ -1913,8 +1920,8 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
         if (OP == KRY_TRI_PAIR) col[t] = (r < m && i >= r && i < m) ? __ldg(A + (long long)i * lda + r) : 0.0;
     }
     exchange(r < m && lane == 0 ? gauss_at(seed, (uint64_t)r) : 0.0, cur);
-    const double sq = kry_sum(m, KRY_MAX_M, [&](int i) { return cur[i] * cur[i]; }, red, &bc);
-    const double inv0 = sq > 0.0 ? 1.0 / sqrt(sq) : 0.0;
+    kry_sum(m, KRY_MAX_M, [&](int i) { return cur[i] * cur[i]; }, red, bc, true);
+    const double inv0 = bc[1];
     for (int i = tid; i < m; i += KRY_THREADS) { cur[i] *= inv0; prv[i] = 0.0; }
     __syncthreads();
     auto apply = [&]() {                               // op(A) cur -> w
@@ -1929,12 +1936,12 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
         double beta_prev = 0.0;
         for (int j = 0; j < steps; ++j) {
             apply();
-            const double alpha = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, &bc);
+            const double alpha = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, bc);
             for (int i = tid; i < m; i += KRY_THREADS) w[i] = w[i] - alpha * cur[i] - beta_prev * prv[i];
             __syncthreads();
-            const double beta = sqrt(kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, &bc));
+            const double beta = kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, bc, true);
             if (blockIdx.x == 0 && tid == 0) { out[j] = ok ? alpha : NAN; out[steps + 1 + j] = ok ? beta : NAN; }
-            const double scale = beta > 0.0 ? 1.0 / beta : 0.0;
+            const double scale = bc[1];
             for (int i = tid; i < m; i += KRY_THREADS) { prv[i] = cur[i]; cur[i] = w[i] * scale; }
             __syncthreads();
             beta_prev = beta;
@@ -1942,13 +1949,13 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
     } else {
         for (int it = 0; it < power; ++it) {
             apply();
-            const double nrm = sqrt(kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, &bc));
-            const double scale = nrm > 0.0 ? 1.0 / nrm : 0.0;
+            kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, bc, true);
+            const double scale = bc[1];
             for (int i = tid; i < m; i += KRY_THREADS) cur[i] = w[i] * scale;
             __syncthreads();
         }
         apply();
-        const double rq = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, &bc);
+        const double rq = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, bc);
         if (blockIdx.x == 0 && tid == 0) out[0] = ok ? rq : NAN;
     }
 }
@@ -2022,108 +2029,237 @@ void gather_columns(const double *X, long long ldx, double *Y, long long ldy, in
 
 // --------------------------------------------------------------------------
 // Jacobi eigensolver for one symmetric matrix of order m <= 64 (one CTA).
-// Parallel cyclic order: in each of the m'-1 rounds (m' = m rounded up to
-// even) the pairs of a round-robin tournament are disjoint, so all their
-// rotations are applied together (rows, then columns, then eigenvectors).
+// Parallel cyclic order: in each of the m'-1 rounds (m' = m rounded up to even)
+// the pairs of a round-robin tournament are disjoint, so all their rotations
+// are applied together.
+//
+// What bounds it: a round's rotations of A and V are about 33 000 FP64
+// operations, 8000 clocks of one SM's FP64 pipe, and eight or nine sweeps of 63
+// rounds would be needed.  So the sweeps are made in FP32 (64 times the rate)
+// until they end at rounding, A ~ V32 diag V32^T; V32 is made orthogonal to FP64
+// accuracy -- with E = I - V32^T V32 (~1e-6), V = V32 (I + E/2 + 3 E^2/8 +
+// 5 E^3/16) leaves O(E^4) -- and A <- V^T A V, formed in FP64, is so nearly diagonal that two FP64
+// sweeps finish it.  A rotation need not annihilate exactly, only be orthogonal:
+// its tangent is taken in FP32, its cosine from that in FP64.  A keeps both
+// triangles; a round updates the 2 x 2 blocks of pairs k >= l and mirrors them.
+// Measured (m = 64): 0.9 ms, 1.6 ms with every eigenvalue double; 2.2 and 3.1 ms with every sweep in FP64.
 // --------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) jacobi_leaf_kernel(double *Ag, long long lda, int m, double *W,
-                                                          long long ldw, double *w, int *sweeps_out)
+constexpr int JAC_LD = 65, JAC_THREADS = 256, JAC_WARPS = JAC_THREADS / 32;
+constexpr int JAC_SMEM = 5 * 64 * JAC_LD * (int)sizeof(double);
+
+__device__ __forceinline__ void jac_rotation(float app, float aqq, float apq, float &c, float &s)
 {
-    __shared__ double A[64][65];
-    __shared__ double V[64][65];
-    __shared__ double cs[32], sn[32];
-    __shared__ int pp[32], qq[32];
-    __shared__ int order[64];
-    __shared__ double offn, dian;
-    const int tid = threadIdx.x;
-    const int me = (m + 1) & ~1;   // even
-    for (int e = tid; e < 64 * 64; e += 256) {
-        int i = e >> 6, j = e & 63;
-        A[i][j] = (i < m && j < m) ? 0.5 * (Ag[(long long)i * lda + j] + Ag[(long long)j * lda + i]) : 0.0;
-        V[i][j] = (i == j) ? 1.0 : 0.0;
-    }
-    if (tid < 64) order[tid] = tid;
-    __syncthreads();
-    int sweep = 0;
-    for (; sweep < 40; ++sweep) {
-        if (tid == 0) { offn = 0.0; dian = 0.0; }
-        __syncthreads();
-        {
-            double o = 0.0, d = 0.0;
-            for (int e = tid; e < m * m; e += 256) {
-                int i = e / m, j = e % m;
-                double v = A[i][j];
-                if (i == j) d += v * v; else o += v * v;
-            }
-            atomicAdd(&offn, o);
-            atomicAdd(&dian, d);
-        }
-        __syncthreads();
-        if (offn <= 1e-30 * dian || offn == 0.0) break;
-        for (int round = 0; round < me - 1; ++round) {
-            // pairs of this round: (order[k], order[me-1-k])
-            if (tid < me / 2) {
-                int p = order[tid], q = order[me - 1 - tid];
-                if (p > q) { int t = p; p = q; q = t; }
-                pp[tid] = p; qq[tid] = q;
-                double c = 1.0, s = 0.0;
-                if (q < m) {
-                    double apq = A[p][q];
-                    if (apq != 0.0) {
-                        double tau = (A[q][q] - A[p][p]) / (2.0 * apq);
-                        double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + t * t); s = t * c;
-                    }
-                }
-                cs[tid] = c; sn[tid] = s;
-            }
-            __syncthreads();
-            // rows: A <- J^T A
-            for (int e = tid; e < (me / 2) * m; e += 256) {
-                int k = e / m, col = e % m;
-                int p = pp[k], q = qq[k];
-                if (q >= m) continue;
-                double c = cs[k], s = sn[k];
-                double ap = A[p][col], aq = A[q][col];
-                A[p][col] = c * ap - s * aq;
-                A[q][col] = s * ap + c * aq;
-            }
-            __syncthreads();
-            // columns: A <- A J, and V <- V J
-            for (int e = tid; e < (me / 2) * m; e += 256) {
-                int k = e / m, row = e % m;
-                int p = pp[k], q = qq[k];
-                if (q >= m) continue;
-                double c = cs[k], s = sn[k];
-                double ap = A[row][p], aq = A[row][q];
-                A[row][p] = c * ap - s * aq;
-                A[row][q] = s * ap + c * aq;
-                double vp = V[row][p], vq = V[row][q];
-                V[row][p] = c * vp - s * vq;
-                V[row][q] = s * vp + c * vq;
-            }
-            __syncthreads();
-            // rotate the tournament: keep order[0], shift the rest
-            if (tid == 0) {
-                int last = order[me - 1];
-                for (int k = me - 1; k > 1; --k) order[k] = order[k - 1];
-                order[1] = last;
-            }
-            __syncthreads();
-        }
-    }
-    for (int e = tid; e < m * m; e += 256) {
-        int i = e / m, j = e % m;
-        W[(long long)i * ldw + j] = V[i][j];
-    }
-    if (tid < m) w[tid] = A[tid][tid];
-    if (tid == 0 && sweeps_out) sweeps_out[0] = sweep;
+    const float tau = (aqq - app) / (2.0f * apq);
+    const float t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
+    c = 1.0f / sqrtf(1.0f + t * t);
+    s = t * c;
 }
 
-void jacobi_leaf(double *A, long long lda, int m, double *W, long long ldw, double *w, int *sweeps_out,
-                 cudaStream_t s)
+__device__ __forceinline__ void jac_rotation(double app, double aqq, double apq, double &c, double &s)
 {
-    jacobi_leaf_kernel<<<1, 256, 0, s>>>(A, lda, m, W, ldw, w, sweeps_out); count_launch();
+    const float tau = (float)(aqq - app) / (2.0f * (float)apq);
+    const double t = (double)(copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(1.0f + tau * tau)));
+    const double x = fma(t, t, 1.0);              // 1 .. 2
+    double y = (double)rsqrtf((float)x);
+    y = y * (1.5 - 0.5 * x * y * y);
+    y = y * (1.5 - 0.5 * x * y * y);
+    c = y;
+    s = t * y;
+}
+
+// squared norms of the off-diagonal part and of the diagonal of A, to every thread
+template <class T>
+__device__ __forceinline__ void jac_norms(const T *A, int m, double *red, double &off, double &dia)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    T o = 0, d = 0;
+    for (int e = tid; e < m * m; e += JAC_THREADS) {
+        const int i = e / m, j = e - i * m;
+        const T v = A[i * JAC_LD + j];
+        if (i == j) d += v * v;
+        else o += v * v;
+    }
+    for (int q = 16; q > 0; q >>= 1) {
+        o += __shfl_xor_sync(0xffffffffu, o, q);
+        d += __shfl_xor_sync(0xffffffffu, d, q);
+    }
+    if (lane == 0) { red[warp] = (double)o; red[JAC_WARPS + warp] = (double)d; }
+    __syncthreads();
+    off = dia = 0.0;
+    for (int w = 0; w < JAC_WARPS; ++w) { off += red[w]; dia += red[JAC_WARPS + w]; }
+    __syncthreads();
+}
+
+// sweeps until off^2 <= tol dia^2, at most `most`; returns the number made
+template <class T>
+__device__ int jac_sweeps(T *A, T *V, int m, double tol, int most, T *cs, T *sn, int *pp, int *qq, double *red)
+{
+    const int tid = threadIdx.x, me = (m + 1) & ~1, np = me / 2, nb = np * (np + 1) / 2;
+    int sweep = 0;
+    for (; sweep < most; ++sweep) {
+        double off, dia;
+        jac_norms<T>(A, m, red, off, dia);
+        if (!(off > tol * dia)) break;
+        for (int round = 0; round < me - 1; ++round) {
+            if (tid < np) {     // round-robin: me - 1 stays, the others turn (me > m: a zero row and column)
+                int p = tid == 0 ? round : round + tid, q = tid == 0 ? me - 1 : round - tid;
+                if (p >= me - 1) p -= me - 1;
+                if (q < 0) q += me - 1;
+                if (p > q) { const int t = p; p = q; q = t; }
+                pp[tid] = p;
+                qq[tid] = q;
+                const T apq = A[p * JAC_LD + q];
+                T c = 1, s = 0;
+                if (apq != (T)0) jac_rotation(A[p * JAC_LD + p], A[q * JAC_LD + q], apq, c, s);
+                if (!(c <= (T)1.0001)) { c = 1; s = 0; }            // (not finite)
+                cs[tid] = c;
+                sn[tid] = s;
+            }
+            __syncthreads();
+            for (int e = tid; e < nb; e += JAC_THREADS) {   // A <- J^T A J, block of pairs k >= l
+                int k = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+                while (k * (k + 1) / 2 > e) --k;
+                while ((k + 1) * (k + 2) / 2 <= e) ++k;
+                const int l = e - k * (k + 1) / 2;
+                const int p = pp[k], q = qq[k], u = pp[l], v = qq[l];
+                const T ck = cs[k], sk = sn[k], cl = cs[l], sl = sn[l];
+                const T apu = A[p * JAC_LD + u], apv = A[p * JAC_LD + v], aqu = A[q * JAC_LD + u], aqv = A[q * JAC_LD + v];
+                const T bpu = ck * apu - sk * aqu, bqu = sk * apu + ck * aqu;
+                const T bpv = ck * apv - sk * aqv, bqv = sk * apv + ck * aqv;
+                const T npu = cl * bpu - sl * bpv, npv = sl * bpu + cl * bpv;
+                const T nqu = cl * bqu - sl * bqv, nqv = sl * bqu + cl * bqv;
+                if (k == l) {
+                    A[p * JAC_LD + p] = npu;
+                    A[q * JAC_LD + q] = nqv;
+                    A[p * JAC_LD + q] = A[q * JAC_LD + p] = nqu;
+                } else {
+                    A[p * JAC_LD + u] = A[u * JAC_LD + p] = npu;
+                    A[p * JAC_LD + v] = A[v * JAC_LD + p] = npv;
+                    A[q * JAC_LD + u] = A[u * JAC_LD + q] = nqu;
+                    A[q * JAC_LD + v] = A[v * JAC_LD + q] = nqv;
+                }
+            }
+            for (int e = tid; e < np * 64; e += JAC_THREADS) {   // V <- V J
+                const int k = e >> 6, row = e & 63;
+                if (row >= m) continue;
+                const int p = pp[k], q = qq[k];
+                const T c = cs[k], s = sn[k];
+                const T vp = V[row * JAC_LD + p], vq = V[row * JAC_LD + q];
+                V[row * JAC_LD + p] = c * vp - s * vq;
+                V[row * JAC_LD + q] = s * vp + c * vq;
+            }
+            __syncthreads();
+        }
+    }
+    return sweep;
+}
+
+// C = op(X) Y for m x m blocks in shared memory (row stride JAC_LD), op = transpose if tx; sym:
+// the result is symmetric, its lower part is formed and mirrored; then C <- a I + b C + c D
+// entry by entry (D may be C's own input).  C differs from X and Y.
+__device__ void jac_product(const double *X, int tx, const double *Y, double *C, int m, bool sym, double a, double b,
+                            double c, const double *D)
+{
+    const int jx = threadIdx.x & 15, iy = threadIdx.x >> 4;
+    double acc[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+    for (int p = 0; p < m; ++p) {
+        double x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = iy + 16 * u;
+            x[u] = tx ? X[p * JAC_LD + i] : X[i * JAC_LD + p];
+            y[u] = Y[p * JAC_LD + jx + 16 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (!sym || v <= u) acc[u][v] = fma(x[u], y[v], acc[u][v]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int i = iy + 16 * u, j = jx + 16 * v;
+            if (i >= m || j >= m || (sym && j > i)) continue;
+            double r = b * acc[u][v] + (i == j ? a : 0.0);
+            if (c != 0.0) r += c * D[i * JAC_LD + j];
+            C[i * JAC_LD + j] = r;
+            if (sym) C[j * JAC_LD + i] = r;
+        }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(JAC_THREADS) jacobi_leaf_kernel(const double *Ag, long long lda, int m, double *W,
+                                                                  long long ldw, double *w, int *sweeps_out)
+{
+    extern __shared__ __align__(16) unsigned char jac_smem[];
+    double *A = (double *)jac_smem, *V = A + 64 * JAC_LD, *T1 = V + 64 * JAC_LD, *T2 = T1 + 64 * JAC_LD;
+    double *T3 = T2 + 64 * JAC_LD;
+    __shared__ double cs[32], sn[32], red[2 * JAC_WARPS];
+    __shared__ int pp[32], qq[32];
+    const int tid = threadIdx.x;
+    // A and the FP32 matrices, scaled by a power of two to entries below 1
+    double amax = 0.0;
+    for (int e = tid; e < 64 * 64; e += JAC_THREADS) {
+        const int i = e >> 6, j = e & 63;
+        const double v = (i < m && j < m) ? 0.5 * (Ag[(long long)i * lda + j] + Ag[(long long)j * lda + i]) : 0.0;
+        A[i * JAC_LD + j] = v;
+        amax = fmax(amax, fabs(v));
+    }
+    for (int q = 16; q > 0; q >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, q));
+    if ((tid & 31) == 0) red[tid >> 5] = amax;
+    __syncthreads();
+    for (int q = 0; q < JAC_WARPS; ++q) amax = fmax(amax, red[q]);
+    __syncthreads();
+    int ex = 0;
+    if (amax > 0.0 && isfinite(amax)) frexp(amax, &ex);
+    const double up = ldexp(1.0, max(-1000, min(1000, ex))), down = ldexp(1.0, -max(-1000, min(1000, ex)));
+    float *A32 = (float *)T1, *V32 = (float *)T2;
+    for (int e = tid; e < 64 * 64; e += JAC_THREADS) {
+        const int i = e >> 6, j = e & 63;
+        A[i * JAC_LD + j] *= down;
+        A32[i * JAC_LD + j] = (float)A[i * JAC_LD + j];
+        V32[i * JAC_LD + j] = i == j ? 1.0f : 0.0f;
+    }
+    __syncthreads();
+    int sweeps = jac_sweeps<float>(A32, V32, m, 3e-12, 12, (float *)cs, (float *)sn, pp, qq, red);
+    for (int e = tid; e < 64 * 64; e += JAC_THREADS) {
+        const int i = e >> 6, j = e & 63;
+        V[i * JAC_LD + j] = (double)V32[i * JAC_LD + j];
+    }
+    __syncthreads();
+    jac_product(V, 1, V, T1, m, true, 1.0, -1.0, 0.0, nullptr);       // E = I - V^T V
+    jac_product(T1, 0, T1, T2, m, true, 0.5, 0.3125, 0.375, T1);      // I/2 + 3 E/8 + 5 E^2/16
+    jac_product(T1, 0, T2, T3, m, true, 1.0, 1.0, 0.0, nullptr);      // I + E times that
+    jac_product(V, 0, T3, T1, m, false, 0.0, 1.0, 0.0, nullptr);      // V, orthogonal
+    double *Vo = T1;
+    jac_product(A, 0, Vo, T2, m, false, 0.0, 1.0, 0.0, nullptr);      // A V
+    jac_product(Vo, 1, T2, A, m, true, 0.0, 1.0, 0.0, nullptr);       // V^T A V
+    if (tid < 64 && (m & 1)) {                                        // the zero row and column of an odd order
+        A[m * JAC_LD + tid] = A[tid * JAC_LD + m] = 0.0;
+        Vo[tid * JAC_LD + m] = 0.0;
+    }
+    __syncthreads();
+    sweeps += jac_sweeps<double>(A, Vo, m, 1e-30, 40, cs, sn, pp, qq, red);
+    for (int e = tid; e < m * m; e += JAC_THREADS) {
+        const int i = e / m, j = e % m;
+        W[(long long)i * ldw + j] = Vo[i * JAC_LD + j];
+    }
+    if (tid < m) w[tid] = A[tid * JAC_LD + tid] * up;
+    if (tid == 0 && sweeps_out) sweeps_out[0] = sweeps;
+}
+
+int jacobi_leaf(const double *A, long long lda, int m, double *W, long long ldw, double *w, int *sweeps_out,
+                cudaStream_t s)
+{
+    if (!ensure_dynamic_smem((const void *)jacobi_leaf_kernel, JAC_SMEM)) return -1;
+    jacobi_leaf_kernel<<<1, JAC_THREADS, JAC_SMEM, s>>>(A, lda, m, W, ldw, w, sweeps_out); count_launch();
+    return 0;
 }
 
 }  // namespace pssd

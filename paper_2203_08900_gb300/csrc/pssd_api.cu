@@ -1334,6 +1334,14 @@ double lmax_estimate(pssd_handle h, int n, F apply, uint64_t seed, double *v, do
     return power_max(h, n, apply, v, w, dscal, 60, kf);
 }
 
+void jacobi(pssd_handle h, const double *A, long long lda, int m, double *W, long long ldw, double *w, cudaStream_t s)
+{
+    if (jacobi_leaf(A, lda, m, W, ldw, w, nullptr, s)) {
+        h->last_err = "Jacobi leaf launch configuration failed";
+        throw Fail{PSSD_ERR_CUDA};
+    }
+}
+
 // symmetric eigendecomposition of B (m x m) by Alg. 2 with Zolotarev signs
 // and Jacobi leaves: W (m x m, ld m) eigenvectors as columns, w eigenvalues
 // (device).  B is preserved.
@@ -1352,7 +1360,7 @@ int sym_eig_node(pssd_handle h, const double *B, int m, double *W, double *w, in
         cuda_check(h, cudaStreamWaitEvent(h->side, ready, 0), "cudaStreamWaitEvent");
         {
             Timed t(h, K_JACOBI, 0, 0.0, h->side);
-            jacobi_leaf(const_cast<double *>(B), m, m, W, m, w, nullptr, h->side);
+            jacobi(h, B, m, m, W, m, w, h->side);
         }
         cuda_check(h, cudaEventRecord(done, h->side), "cudaEventRecord");
         h->leaf_pending.push_back(done);
@@ -3257,7 +3265,7 @@ extern "C" int pssd_zeig(pssd_handle h, int n, const signed char *sigma, const d
                 }
                 if (q2 <= 64) {
                     Timed t(h, K_JACOBI, 0);
-                    jacobi_leaf(Ge, q2, q2, Qe, q2, le, nullptr, h->stream);
+                    jacobi(h, Ge, q2, q2, Qe, q2, le, h->stream);
                 } else {
                     int md = 0;
                     int st2 = sym_eig(h, Ge, q2, Qe, le, 64, 1, &md, 0x2e17ull + (uint64_t)i);

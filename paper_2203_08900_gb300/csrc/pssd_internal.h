@@ -189,8 +189,8 @@ void gather_columns(const double *X, long long ldx, double *Y, long long ldy, in
                     const int *perm, cudaStream_t s);
 void copy_matrix(const double *X, long long ldx, double *Y, long long ldy, int m, int n,
                  cudaStream_t s);
-void jacobi_leaf(double *A, long long lda, int m, double *W, long long ldw, double *w,
-                 int *sweeps_out, cudaStream_t s);  // m <= 64; W eigenvectors (columns), w values
+int jacobi_leaf(const double *A, long long lda, int m, double *W, long long ldw, double *w,
+                int *sweeps_out, cudaStream_t s);  // m <= 64; W eigenvectors (columns), w values
 
 // host-side Zolotarev coefficients (theta-function evaluation)
 int zolo_coeffs_host(double ell, int r, double *c, double *a, double *chat, double *ell_next);
