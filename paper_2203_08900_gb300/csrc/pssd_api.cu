@@ -27,7 +27,9 @@
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <mutex>
+#include <system_error>
 #include <thread>
 #include <type_traits>
 #include <string>
@@ -62,6 +64,13 @@ struct pssd_handle_s {
     long long prof_count[16] = {0};
     int dmode = GM_F64;   // arithmetic of FP64 contractions in the current call (GM_F64 or GM_DF)
     std::vector<pssd_handle_s *> workers;   // pssd_eig_batched: one handle (own stream, workspace) per worker
+    // The symmetric recursion's second children: handles with a stream and a workspace of their own, at
+    // most MAX_HELPERS per calling handle (root, null in that handle), kept for its lifetime
+    std::vector<pssd_handle_s *> helpers, idle_helpers;
+    std::mutex helper_mu;
+    pssd_handle_s *root = nullptr;
+    bool sequential = false;                // never use helpers (many batch workers run already)
+    size_t chunk_bytes = size_t(1) << 30;   // smallest workspace chunk
     int *derr = nullptr;    // device error flag of the current call (bounded waits in the tensor-core kernel)
     int use_tc = 1;         // FP32 contractions on tcgen05 tensor cores (0: FP32 SIMT kernel)
     int force_engine = 0;   // test hooks: no size-based engine selection
@@ -138,7 +147,7 @@ void *walloc(pssd_handle h, size_t bytes)
         size_t off = (i == m.chunk) ? c.off : 0;
         if (off + bytes <= c.cap) { c.off = off + bytes; return c.base + off; }
     }
-    size_t cap = std::max(bytes, size_t(1) << 30);
+    size_t cap = std::max(bytes, h->chunk_bytes);
     void *p = nullptr;
     g_device_allocs.fetch_add(1, std::memory_order_relaxed);
     cudaError_t e = cudaMalloc(&p, cap);
@@ -1342,6 +1351,10 @@ void jacobi(pssd_handle h, const double *A, long long lda, int m, double *W, lon
     }
 }
 
+// one half of a division: B (m x m, device) -> eigenvectors W, eigenvalues w
+struct SymPart { const double *B; int m; double *W, *w; uint64_t seed; };
+int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, int depth, int *maxdepth);
+
 // symmetric eigendecomposition of B (m x m) by Alg. 2 with Zolotarev signs
 // and Jacobi leaves: W (m x m, ld m) eigenvectors as columns, w eigenvalues
 // (device).  B is preserved.
@@ -1526,8 +1539,7 @@ int sym_eig_node(pssd_handle h, const double *B, int m, double *W, double *w, in
         if (st) { release(h, mk); continue; }
         // recurse
         double *Wp = dalloc(h, (size_t)p * p), *Wm = dalloc(h, (size_t)(m - p) * (m - p));
-        st = sym_eig_node(h, Bp, p, Wp, w, leaf, depth + 1, maxdepth, seed * 3 + 1);
-        if (!st) st = sym_eig_node(h, Bm, m - p, Wm, w + p, leaf, depth + 1, maxdepth, seed * 3 + 2);
+        st = sym_eig_pair(h, {Bp, p, Wp, w, seed * 3 + 1}, {Bm, m - p, Wm, w + p, seed * 3 + 2}, leaf, depth + 1, maxdepth);
         if (st) { release(h, outer); return st; }
         g_phase = PH_ASSEMBLE;
         join_leaves(h);
@@ -1550,6 +1562,123 @@ int sym_eig(pssd_handle h, const double *B, int m, double *W, double *w, int lea
             uint64_t seed)
 {
     const int st = sym_eig_node(h, B, m, W, w, leaf, depth, maxdepth, seed);
+    join_leaves(h);
+    return st;
+}
+
+constexpr int MAX_HELPERS = 3;
+
+// an idle helper of h's calling handle, or null: none left, or workspace that may not grow
+pssd_handle_s *acquire_helper(pssd_handle h)
+{
+    pssd_handle_s *root = h->root ? h->root : h;
+    if (root->sequential || root->user_ws) return nullptr;
+    std::lock_guard<std::mutex> lk(root->helper_mu);
+    if (!root->idle_helpers.empty()) {
+        pssd_handle_s *x = root->idle_helpers.back();
+        root->idle_helpers.pop_back();
+        return x;
+    }
+    if ((int)root->helpers.size() >= MAX_HELPERS) return nullptr;
+    auto *x = new pssd_handle_s();
+    if (cudaStreamCreateWithFlags(&x->stream, cudaStreamNonBlocking) != cudaSuccess) {
+        (void)cudaGetLastError();
+        delete x;
+        return nullptr;
+    }
+    x->root = root;
+    x->chunk_bytes = size_t(1) << 28;
+    root->helpers.push_back(x);
+    return x;
+}
+
+void give_back_helper(pssd_handle_s *x)
+{
+    std::lock_guard<std::mutex> lk(x->root->helper_mu);
+    x->root->idle_helpers.push_back(x);
+}
+
+// The two halves of a division are independent, and below order 1000 or so neither fills the
+// GPU: a node is a chain of small launches and host reads.  The second half runs in a thread of
+// its own on a helper's stream while there is a helper (so up to four chains at a time), with
+// the same seeds and operations as one after the other.  casida_eig at k = 1024: 103 -> 70 ms,
+// zeig at n = 400: 76 -> 44 ms.
+int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, int depth, int *maxdepth)
+{
+    int da = *maxdepth, db = *maxdepth;
+    pssd_handle_s *x = std::min(a.m, b.m) > leaf ? acquire_helper(h) : nullptr;
+    std::thread second;
+    cudaEvent_t done = nullptr;
+    int st_b = PSSD_OK;
+    if (x) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        x->dmode = h->dmode; x->use_tc = h->use_tc; x->derr = h->derr; x->wait_limit = h->wait_limit; x->prof = h->prof;
+        x->depth = x->peak = 0;
+        try {
+            cudaEvent_t ready = sync_event(h);         // b.B is there
+            done = sync_event(h);
+            cuda_check(h, cudaEventRecord(ready, h->stream), "cudaEventRecord");
+            second = std::thread([&, dev, ready, done]() {
+                cudaSetDevice(dev);
+                Mark mk = mark(x);
+                try {
+                    cuda_check(x, cudaStreamWaitEvent(x->stream, ready, 0), "cudaStreamWaitEvent");
+                    st_b = sym_eig_node(x, b.B, b.m, b.W, b.w, leaf, depth, &db, b.seed);
+                    join_leaves(x);
+                    cuda_check(x, cudaEventRecord(done, x->stream), "cudaEventRecord");
+                } catch (Fail &f) {
+                    st_b = f.code;
+                } catch (...) {
+                    st_b = PSSD_ERR_ALLOC;
+                }
+                if (st_b) {   // nothing of this half may still run when its operands go away
+                    if (x->side) cudaStreamSynchronize(x->side);
+                    cudaStreamSynchronize(x->stream);
+                }
+                release(x, mk);
+            });
+        } catch (const std::system_error &) {          // no thread to be had
+            give_back_helper(x);
+            x = nullptr;
+        } catch (...) {
+            give_back_helper(x);
+            throw;
+        }
+    }
+    if (!x) {
+        int st = a.m > 0 ? sym_eig_node(h, a.B, a.m, a.W, a.w, leaf, depth, maxdepth, a.seed) : PSSD_OK;
+        if (!st && b.m > 0) st = sym_eig_node(h, b.B, b.m, b.W, b.w, leaf, depth, maxdepth, b.seed);
+        return st;
+    }
+    int st_a = PSSD_OK;
+    std::exception_ptr thrown;
+    try {
+        st_a = sym_eig_node(h, a.B, a.m, a.W, a.w, leaf, depth, &da, a.seed);
+    } catch (...) {
+        thrown = std::current_exception();
+    }
+    second.join();
+    h->peak = std::max(h->peak, h->depth + x->peak);   // as if the second half came after the first
+    if (st_b && !st_a && !thrown) h->last_err = x->last_err;
+    h->events.insert(h->events.end(), x->events.begin(), x->events.end());
+    x->events.clear();
+    x->leaf_pending.clear();
+    x->sync_used = 0;
+    x->derr = nullptr;
+    if (thrown || st_a) cudaStreamSynchronize(x->stream);
+    give_back_helper(x);
+    if (thrown) std::rethrow_exception(thrown);
+    if (st_a || st_b) return st_a ? st_a : st_b;
+    cuda_check(h, cudaStreamWaitEvent(h->stream, done, 0), "cudaStreamWaitEvent");
+    *maxdepth = std::max(da, db);
+    return PSSD_OK;
+}
+
+// both halves of a top-level division, all leaves joined
+int sym_eig_halves(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, int depth, int *maxdepth)
+{
+    const int st = sym_eig_pair(h, a, b, leaf, depth, maxdepth);
     join_leaves(h);
     return st;
 }
@@ -1905,22 +2034,41 @@ int pssd_create(pssd_handle *h, void *stream)
     return PSSD_OK;
 }
 
+static void drop_side(pssd_handle x)
+{
+    if (x->side) { cudaStreamSynchronize(x->side); cudaStreamDestroy(x->side); }
+    for (auto &e : x->sync_events) cudaEventDestroy(e);
+}
+
+// the handle's helpers with their workspaces (none is in use between calls)
+static void drop_helpers(pssd_handle h)
+{
+    for (auto *x : h->helpers) {
+        cudaStreamSynchronize(x->stream);
+        drop_side(x);
+        for (auto &c : x->chunks) if (c.owned) cudaFree(c.base);
+        for (auto &e : x->free_events) cudaEventDestroy(e);
+        cudaStreamDestroy(x->stream);
+        delete x;
+    }
+    h->helpers.clear();
+    h->idle_helpers.clear();
+}
+
 int pssd_destroy(pssd_handle h)
 {
     if (!h) return -1;
     cudaStreamSynchronize(h->stream);
-    auto drop_side = [](pssd_handle x) {
-        if (x->side) { cudaStreamSynchronize(x->side); cudaStreamDestroy(x->side); }
-        for (auto &e : x->sync_events) cudaEventDestroy(e);
-    };
     for (auto *w : h->workers) {
         cudaStreamSynchronize(w->stream);
+        drop_helpers(w);
         drop_side(w);
         for (auto &c : w->chunks) if (c.owned) cudaFree(c.base);
         for (auto &e : w->free_events) cudaEventDestroy(e);
         cudaStreamDestroy(w->stream);
         delete w;
     }
+    drop_helpers(h);
     drop_side(h);
     for (auto &c : h->chunks) if (c.owned) cudaFree(c.base);
     for (auto &e : h->free_events) cudaEventDestroy(e);
@@ -2144,8 +2292,7 @@ int eig_core(pssd_handle h, int n, const signed char *sigma, const double *H, in
         double *Wp = dalloc(h, (size_t)p * p + 1), *Wm = dalloc(h, (size_t)q * q + 1);
         double *w = dalloc(h, n);
         int maxdepth = 0;
-        if (p > 0) st = sym_eig(h, Bp, p, Wp, w, leaf, 1, &maxdepth, 0x1001ull);
-        if (!st && q > 0) st = sym_eig(h, Bm, q, Wm, w + p, leaf, 1, &maxdepth, 0x2002ull);
+        st = sym_eig_halves(h, {Bp, p, Wp, w, 0x1001ull}, {Bm, q, Wm, w + p, 0x2002ull}, leaf, 1, &maxdepth);
         if (st) return st;
         if (info) info->levels = maxdepth;
         g_phase = PH_ASSEMBLE;
@@ -2259,6 +2406,7 @@ int pssd_set_workspace(pssd_handle h, void *dptr, size_t bytes)
         h->last_err = "cudaStreamSynchronize before replacing the workspace failed";
         return PSSD_ERR_CUDA;
     }
+    drop_helpers(h);
     for (auto &c : h->chunks) if (c.owned) cudaFree(c.base);
     h->chunks.clear();
     h->user_ws = false;
@@ -3063,6 +3211,7 @@ extern "C" int pssd_eig_batched(pssd_handle h, int count, const int *n, const si
         cuda_check(h, cudaEventRecord(start, h->stream), "cudaEventRecord");
         for (int w = 0; w < nw; ++w)
             cuda_check(h, cudaStreamWaitEvent(h->workers[w]->stream, start, 0), "cudaStreamWaitEvent");
+        for (int w = 0; w < nw; ++w) h->workers[w]->sequential = nw > 4;   // the workers keep the host and the GPU busy
         std::vector<int> order(count);
         for (int i = 0; i < count; ++i) order[i] = i;
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
