@@ -2543,9 +2543,11 @@ namespace {
 // the sum of the positive eigenvalues (gradient P_+^T, P_+ = (I + S)/2): the gradient of the
 // computed function, coefficients and bounds held fixed.  Backward of one step
 // X' = chat (X + X T), T = sum_j a_j Z_j, Z_j = (X^2 + c_{2j-1} I)^{-1}:
-//   Abar = chat X X'bar,  B = sum_j a_j Z_j Abar Z_j,
-//   Xbar = chat (X'bar + X'bar T) - (X B + B X)
-// (dZ_j = -Z_j (X dX + dX X) Z_j; X, T, Z_j symmetric and commuting).  Then K = alpha X_0,
+//   Abar = sym(chat X X'bar),  B = sum_j a_j Z_j Abar Z_j,
+//   Xbar = sym(chat (X'bar + X'bar T) - 2 X B)
+// (dZ_j = -Z_j (X dX + dX X) Z_j; X, T, Z_j symmetric and commuting; X is symmetric, so only the
+// symmetric part of Xbar counts, which makes B symmetric and takes one product instead of X B
+// and B X: (6 + 3 r) n^3 flops a step instead of (8 + 4 r) n^3).  Then K = alpha X_0,
 // K = L^T Sigma L gives Lbar += Sigma L (Kbar + Kbar^T); S = L^{-T} Y L^T gives, with
 // Ghat = L^{-1} G L, Ybar = sym(Ghat) and Lbar += L^{-T} (Ghat^T Y - Y Ghat^T); the
 // Cholesky factorisation M = L L^T gives Mbar = sym(L^{-T} Phi(L^T Lbar) L^{-1}) (Phi: lower
@@ -2607,25 +2609,27 @@ int sign_vjp_steps(pssd_handle h, const Front &F, const SignTape &tape, const do
             GemmArgs ga; ga.m = ga.n = ga.k = n; ga.A = stp.X; ga.lda = ld; ga.B = Xb; ga.ldb = ld; ga.C = Ab;
             ga.ldc = ld; ga.alpha = stp.chat;
             gemm(h, ga);                                                       // Abar = chat X Xbar'
+            {   // only sym(Xbar) is used, and sym(X B + B X) = sym(2 X sym B): B from sym(Abar), symmetric
+                Timed t(h, K_HBM, 0, 16.0 * n * (double)n);
+                sym_average<double>(Ab, ld, n, h->stream);
+            }
             for (int j = 0; j < r; ++j) {
                 const double *Zj = Z + (long long)j * nsz;
                 GemmArgs g1; g1.m = g1.n = g1.k = n; g1.A = Zj; g1.lda = ld; g1.B = Ab; g1.ldb = ld; g1.C = W1;
                 g1.ldc = ld;
                 gemm(h, g1);                                                   // Z_j Abar
                 GemmArgs g2; g2.m = g2.n = g2.k = n; g2.A = W1; g2.lda = ld; g2.B = Zj; g2.ldb = ld; g2.C = Bs;
-                g2.ldc = ld; g2.alpha = stp.a[j];
+                g2.ldc = ld; g2.alpha = stp.a[j]; g2.lowerC = 1;
                 if (j) { g2.Cin = Bs; g2.ldcin = ld; g2.beta = 1.0; }
-                gemm(h, g2);                                                   // B += a_j Z_j Abar Z_j
+                gemm(h, g2);                                                   // B += a_j Z_j Abar Z_j (lower)
             }
+            mirror<double>(h, Bs, ld, 0, n, 1);
             GemmArgs gx; gx.m = gx.n = gx.k = n; gx.A = Xb; gx.lda = ld; gx.B = Tm; gx.ldb = ld; gx.Cin = Xb;
             gx.ldcin = ld; gx.C = Xn; gx.ldc = ld; gx.alpha = stp.chat; gx.beta = stp.chat;
             gemm(h, gx);                                                       // chat (Xbar' + Xbar' T)
             GemmArgs g3; g3.m = g3.n = g3.k = n; g3.A = stp.X; g3.lda = ld; g3.B = Bs; g3.ldb = ld; g3.Cin = Xn;
-            g3.ldcin = ld; g3.C = Xn; g3.ldc = ld; g3.alpha = -1.0; g3.beta = 1.0;
-            gemm(h, g3);                                                       // - X B
-            GemmArgs g4; g4.m = g4.n = g4.k = n; g4.A = Bs; g4.lda = ld; g4.B = stp.X; g4.ldb = ld; g4.Cin = Xn;
-            g4.ldcin = ld; g4.C = Xn; g4.ldc = ld; g4.alpha = -1.0; g4.beta = 1.0;
-            gemm(h, g4);                                                       // - B X
+            g3.ldcin = ld; g3.C = Xn; g3.ldc = ld; g3.alpha = -2.0; g3.beta = 1.0;
+            gemm(h, g3);                                                       // - 2 X B (its symmetric part is taken above)
             std::swap(Xb, Xn);
             release(h, ms);
         }
