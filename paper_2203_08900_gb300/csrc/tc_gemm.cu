@@ -265,13 +265,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
 // (p % 16) / 4 is stored at chunk ((p % 16) / 4) ^ ((rr / 2) % 4) (the
 // 64-byte shared-memory swizzle the MMA descriptors expect).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) tf32_split_kernel(const float *X, long long ld, long long sb, int trans,
-                                                         int rows, int k, int k_pad, int rows_pad, int tile_rows,
-                                                         int tri, const float *ks, float *out)
+// One operand: op(X) is rows x k (trans: op(X)[r][p] = X[p][r]), tri and ks as above.
+struct TcOperand {
+    const float *X; long long ld, sb; int trans, rows, rows_pad, tile_rows, tri; const float *ks; float *out;
+};
+
+// both operands in one launch: grid rows [0, nA) serve A, the rest B
+__global__ void __launch_bounds__(256) tf32_split_kernel(TcOperand a, TcOperand b, int k, int k_pad, int nA)
 {
+    const bool isA = (int)blockIdx.y < nA;
+    const TcOperand &op = isA ? a : b;
+    const float *X = op.X, *ks = op.ks;
+    const long long ld = op.ld, sb = op.sb;
+    const int trans = op.trans, rows = op.rows, rows_pad = op.rows_pad, tile_rows = op.tile_rows, tri = op.tri;
+    float *out = op.out;
     __shared__ float T[32][33];
     const int z = blockIdx.z;
-    const int r0 = blockIdx.y * 32, p0 = blockIdx.x * 32;
+    const int r0 = (isA ? (int)blockIdx.y : (int)blockIdx.y - nA) * 32, p0 = blockIdx.x * 32;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
     X += (long long)z * sb;
     // load the 32 x 32 block in the orientation that is contiguous in memory
@@ -339,17 +349,12 @@ int tc_gemm_prepare(const GemmArgs &g, void *ws, cudaStream_t s)
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return 0;
     int kp, mp, np; float *ta, *tb;
     tc_layout(g, ws, kp, mp, np, ta, tb);
-    {   // A: rows i of op(A), K-major
-        dim3 grid((kp + 31) / 32, (mp + 31) / 32, g.batch);
-        tf32_split_kernel<<<grid, 256, 0, s>>>((const float *)g.A, g.lda, g.sA, g.ta, g.m, g.k, kp, mp, TC_BM,
-                                               g.triA, (const float *)g.kscale, ta); count_launch();
-    }
-    {   // B: rows j of op(B)^T, K-major (op(B)[p][j] = B[p][j] or B[j][p])
-        int triB = g.triB == TRI_LOWER ? TRI_UPPER : (g.triB == TRI_UPPER ? TRI_LOWER : TRI_NONE);
-        dim3 grid((kp + 31) / 32, (np + 31) / 32, g.batch);
-        tf32_split_kernel<<<grid, 256, 0, s>>>((const float *)g.B, g.ldb, g.sB, g.tb ? 0 : 1, g.n, g.k, kp, np, TC_BN,
-                                               triB, nullptr, tb); count_launch();
-    }
+    // A: rows i of op(A); B: rows j of op(B)^T (op(B)[p][j] = B[p][j] or B[j][p]); both K-major
+    const int triB = g.triB == TRI_LOWER ? TRI_UPPER : (g.triB == TRI_UPPER ? TRI_LOWER : TRI_NONE);
+    const TcOperand oa{(const float *)g.A, g.lda, g.sA, g.ta, g.m, mp, TC_BM, g.triA, (const float *)g.kscale, ta};
+    const TcOperand ob{(const float *)g.B, g.ldb, g.sB, g.tb ? 0 : 1, g.n, np, TC_BN, triB, nullptr, tb};
+    const int nA = mp / 32, nB = np / 32;
+    tf32_split_kernel<<<dim3((kp + 31) / 32, nA + nB, g.batch), 256, 0, s>>>(oa, ob, g.k, kp, nA); count_launch();
     return 0;
 }
 
