@@ -694,140 +694,185 @@ chol_leaf64_kernel(double *A, long long lda, long long sA, double *Rinv, long lo
         }
 }
 
-// ---- FP32: blocks of at most 128 ----
+// ---- FP32: blocks of at most 128, four block columns of 32 ----
+//
+// The same division of work as in FP64: a chain warp that publishes column after column, three
+// warps that bring the later columns up to date in shared memory, three that follow with the
+// inverse.  What bounds it here is latency -- a column's square root, reciprocal and hand-over,
+// about 200 clocks -- and, for code that runs a few times per launch, its fetch: with a block
+// unrolled in the registers of one warp a leaf took 100 us.  Measured (128 x 128): 62 us.
 
-// One warp: lane i holds row i of the block in registers; column j's scaled entries go
-// through a shared-memory buffer (double-buffered by j), and each lane loads the ones it needs
-// before its updates, so the loads pipeline.
-__device__ __forceinline__ void leaf_diag_block_warp(float *Lb, float *Xb, int ls, int w, float *rv, int lane,
-                                                     int *info, int z, int gpiv, int *bad, float *colbuf)
+__device__ __forceinline__ void leaf32_chain(float *Lb, int ls, int w, float *rv, uint32_t done, uint32_t ready,
+                                             int lane, int *info, int z, int gpiv, int *bad)
 {
-    float d[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) d[c] = (lane < w && c <= lane) ? Lb[lane * ls + c] : 0.f;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        if (j < w) {
-            float pj = __shfl_sync(0xffffffffu, d[j], j);
-            if (!(pj > 0.f) || !isfinite(pj)) {
-                if (lane == 0 && !*bad) { *bad = 1; if (info[z] == 0) info[z] = gpiv + j + 1; }
-                pj = 1.f;
-            }
-            float piv, r;
-            LeafPivot::get(pj, piv, r);
-            const float lij = (lane == j) ? piv : ((lane > j) ? d[j] * r : d[j]);
-            d[j] = lij;
-            float *cb = colbuf + (j & 1) * 32;
-            cb[lane] = lij;
-            if (lane == 0) rv[j] = r;
-            __syncwarp();
-            float lc[32];
-#pragma unroll
-            for (int c = j + 1; c < 32; ++c) lc[c] = cb[c];
-#pragma unroll
-            for (int c = j + 1; c < 32; ++c)
-                if (lane >= c) d[c] -= lij * lc[c];
+    float *row = Lb + min(lane, w - 1) * ls;          // (lanes beyond the last row repeat it)
+    float v = 0.f, vc = 0.f, d = row[0], dc = Lb[0];
+    for (int c = 0; c < w; ++c) {
+        float pv = fmaf(-vc, vc, dc);
+        d = fmaf(-v, vc, d);
+        if (!(pv > 0.f) || !isfinite(pv)) {
+            if (lane == 0 && !*bad) { *bad = 1; if (info[z] == 0) info[z] = gpiv + c + 1; }
+            pv = 1.f;
         }
-    }
-#pragma unroll
-    for (int c = 0; c < 32; ++c)
-        if (lane < w && c <= lane) Lb[lane * ls + c] = d[c];
-    __syncwarp();
-    float x[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-        float v = 0.f;
-        if (k < w) {
-            float acc = 0.f;
-#pragma unroll
-            for (int m = 0; m < k; ++m) acc += Lb[k * ls + m] * x[m];
-            v = (k == lane) ? rv[k] : ((k > lane) ? -acc * rv[k] : 0.f);
-        }
-        x[k] = v;
-    }
-    if (lane < w) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-            if (k < w && k >= lane) Xb[k * ls + lane] = x[k];
+        const int cn = min(c + 1, w - 1);
+        float piv, r;
+        LeafPivot::get(pv, piv, r);
+        v = lane == c ? piv : d * r;
+        vc = __shfl_sync(0xffffffffu, v, cn);
+        if (lane >= c && lane < w) row[c] = v;
+        if (lane == 0) rv[c] = r;
+        __syncwarp();
+        mbar_arrive_if(done + 8 * c, lane == 0);
+        if (cn >= 2 && cn > c) mbar_wait(ready + 8 * cn, 0u, LEAF_WAIT_LIMIT);
+        d = row[cn];
+        dc = Lb[cn * ls + cn];
     }
 }
 
-// The s x s diagonal block at (off, off) of batch matrix blockIdx.x, in shared memory (row
-// stride s + 1), factorised right-looking by blocks of 32 columns with 8 warps:
-//   1. warp 0 factorises the diagonal block and inverts it;
+// columns u, u + 3, ...: the columns before their last but one, in turn
+__device__ __forceinline__ void leaf32_update(float *Lb, int ls, int w, uint32_t done, uint32_t ready, int u, int lane)
+{
+    float *row = Lb + min(lane, w - 1) * ls;
+    for (int j = 0; j + 2 < w; ++j) {
+        mbar_wait(done + 8 * j, 0u, LEAF_WAIT_LIMIT);
+        const float li = row[j];
+        for (int c0 = j + 2 + (u + 6 - (j + 2) % 3) % 3; c0 < w; c0 += 12) {
+            float v[4];                               // four columns' loads, then their stores
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int c = min(c0 + 3 * t, w - 1);
+                v[t] = fmaf(-li, Lb[c * ls + j], row[c]);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (c0 + 3 * t < w && lane >= c0 + 3 * t && lane < w) row[c0 + 3 * t] = v[t];
+            if (c0 == j + 2) {
+                __syncwarp();
+                mbar_arrive_if(ready + 8 * c0, lane == 0);
+            }
+        }
+    }
+}
+
+// rows iw, iw + 3, ... of X_D = L_D^{-1}: x_kc = -(sum_m L_km x_mc) / L_kk, m ascending, the
+// sums growing in Xb (zero at first)
+__device__ __forceinline__ void leaf32_invert(const float *Lb, float *Xb, int ls, int w, const float *rv, uint32_t done,
+                                              uint32_t row, int iw, int lane)
+{
+    const int col = min(lane, w - 1);
+    auto finish = [&](int j) {
+        mbar_wait(done + 8 * j, 0u, LEAF_WAIT_LIMIT);
+        const float r = rv[j], acc = Xb[j * ls + col];
+        if (lane < w) Xb[j * ls + lane] = lane < j ? -acc * r : (lane == j ? r : 0.f);
+        __syncwarp();
+        mbar_arrive_if(row + 8 * j, lane == 0);
+    };
+    if (iw == 0) finish(0);
+    for (int j = 0; j + 1 < w; ++j) {
+        mbar_wait(row + 8 * j, 0u, LEAF_WAIT_LIMIT);
+        const float x = Xb[j * ls + col];
+        for (int k0 = j + 1 + (iw + 6 - (j + 1) % 3) % 3; k0 < w; k0 += 12) {
+            float v[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int k = min(k0 + 3 * t, w - 1);
+                v[t] = fmaf(Lb[k * ls + j], x, Xb[k * ls + col]);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (k0 + 3 * t < w && lane < w) Xb[(k0 + 3 * t) * ls + lane] = v[t];
+            if (k0 == j + 1) { __syncwarp(); finish(k0); }
+        }
+    }
+}
+
+// The s x s (s <= 128) diagonal block at (off, off) of batch matrix blockIdx.x, right-looking by
+// blocks of 32 columns with 8 warps:
+//   1. the diagonal block and its inverse X_D (warp 0, warps 1-3, warps 5-7);
 //   2. panel L_21 = A_21 X_D^T: a warp per row of A_21, lane c holding row c of X_D in
 //      registers, the row of A_21 read as shared-memory broadcasts;
 //   3. trailing update A_22 -= L_21 L_21^T: lane j holding rows j, j + 32, j + 64 of L_21 in
-//      registers, a warp per row i, the lower triangle stored;
-// three barriers per block of 32 columns.  Then the off-diagonal blocks of X = L^{-1}, block
-// row i after block row i - 1: X_ik = -X_ii (sum_{m=k}^{i-1} L_im X_mk), all k < i at once,
-// two rows per warp.
+//      registers, a warp per row i, the lower triangle stored.
+// Then the off-diagonal blocks of X = L^{-1}, block row i after block row i - 1:
+// X_ik = -X_ii (sum_{m=k}^{i-1} L_im X_mk), all k < i at once, four rows per warp.
 __global__ void __launch_bounds__(256) chol_leaf128_kernel(float *A, long long lda, long long sA, float *Rinv,
                                                            long long ldr, long long sR, int off, int s, int *info)
 {
     constexpr int NQ = 3;                     // 32-row groups of a panel
-    using T = float;
     extern __shared__ unsigned char leaf_smem[];
-    const int ls = s + 1;
-    T *L = (T *)leaf_smem;                    // the block, then L
-    T *X = L + (size_t)s * ls;                // L^{-1}
-    T *W = X + (size_t)s * ls;                // s x 33: the panel, then block products of the inverse
-    T *rv = W + (size_t)s * 33;               // 1 / L_jj
+    const int ls = s | 1;
+    float *L = (float *)leaf_smem;            // the block, then L
+    float *X = L + (size_t)s * ls;            // L^{-1}
+    float *W = X + (size_t)s * ls;            // s x 33: the panel, then block products of the inverse
+    float *rv = W + (size_t)s * 33;           // 1 / L_jj
     __shared__ int bad;
-    __shared__ T colbuf[64];                  // the FP32 diagonal block's column buffer
+    __shared__ unsigned long long bars[4 * 96];   // per block column: done, ready, rows of X
     const int z = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     A += (long long)z * sA + (long long)off * lda + off;
     Rinv += (long long)z * sR + (long long)off * ldr + off;
     if (tid == 0) bad = 0;
-    for (int r = warp; r < s; r += 8)
-        for (int c = lane; c < s; c += 32) {
-            L[r * ls + c] = (c <= r) ? A[(long long)r * lda + c] : (T)0;
-            X[r * ls + c] = (T)0;
+    for (int e = tid; e < 4 * 96; e += 256) mbar_init(smem_u32(bars + e), 1);
+    for (int e0 = tid; e0 < 128 * 128; e0 += 256 * 16) {   // 16 loads of a thread in flight at once
+        float v[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            const int e = e0 + 256 * t, r = e >> 7, c = e & 127;
+            v[t] = (r < s && c <= r) ? A[(long long)r * lda + c] : 0.f;
         }
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            const int e = e0 + 256 * t, r = e >> 7, c = e & 127;
+            if (r < s && c < s) { L[r * ls + c] = v[t]; X[r * ls + c] = 0.f; }
+        }
+    }
     __syncthreads();
     const int nb = (s + 31) >> 5;
     for (int kb = 0; kb < nb; ++kb) {
         const int o = kb * 32, w = min(32, s - o), o2 = o + w, rows = s - o2;
-        if (warp == 0)
-            leaf_diag_block_warp(L + o * ls + o, X + o * ls + o, ls, w, rv + o, lane, info, z, off + o, &bad, colbuf);
+        {
+            float *Ld = L + o * ls + o;
+            const uint32_t done = smem_u32(bars + 96 * kb), ready = done + 256, row = done + 512;
+            if (warp == 0) leaf32_chain(Ld, ls, w, rv + o, done, ready, lane, info, z, off + o, &bad);
+            else if (warp < 4) leaf32_update(Ld, ls, w, done, ready, warp - 1, lane);
+            else if (warp > 4) leaf32_invert(Ld, X + o * ls + o, ls, w, rv + o, done, row, warp - 5, lane);
+        }
         __syncthreads();
-        if (rows > 0) {
+        if (rows > 0) {                       // (w = 32)
             {   // W[i][c] = sum_{m <= c} A[o2 + i][o + m] X_D[c][m]
-                T xd[32];
+                float xd[32];
 #pragma unroll
-                for (int m = 0; m < 32; ++m) xd[m] = (lane < w && m < w) ? X[(o + lane) * ls + o + m] : (T)0;
+                for (int m = 0; m < 32; ++m) xd[m] = X[(o + lane) * ls + o + m];
                 for (int i = warp; i < rows; i += 8) {
-                    const T *a = L + (o2 + i) * ls + o;
-                    T acc = (T)0;
+                    const float *a = L + (o2 + i) * ls + o;
+                    float acc = 0.f;
 #pragma unroll
-                    for (int m = 0; m < 32; ++m)
-                        if (m < w) acc += a[m] * xd[m];
+                    for (int m = 0; m < 32; ++m) acc += a[m] * xd[m];
                     W[i * 33 + lane] = acc;
                 }
             }
             __syncthreads();
             {
-                T wr[NQ][32];
+                float wr[NQ][32];
 #pragma unroll
                 for (int q = 0; q < NQ; ++q)
 #pragma unroll
                     for (int c = 0; c < 32; ++c) {
                         const int j = lane + 32 * q;
-                        wr[q][c] = (j < rows && c < w) ? W[j * 33 + c] : (T)0;
+                        wr[q][c] = j < rows ? W[j * 33 + c] : 0.f;
                     }
                 for (int i = warp; i < rows; i += 8) {
-                    const T *wi = W + i * 33;
-                    T acc[NQ];
+                    const float *wi = W + i * 33;
+                    float acc[NQ];
 #pragma unroll
-                    for (int q = 0; q < NQ; ++q) acc[q] = (T)0;
+                    for (int q = 0; q < NQ; ++q) acc[q] = 0.f;
 #pragma unroll
                     for (int c = 0; c < 32; ++c) {
-                        const T v = wi[c];
+                        const float v = wi[c];
 #pragma unroll
                         for (int q = 0; q < NQ; ++q) acc[q] += v * wr[q][c];
                     }
-                    T *lrow = L + (o2 + i) * ls;
-                    if (lane < w) lrow[o + lane] = wi[lane];
+                    float *lrow = L + (o2 + i) * ls;
+                    lrow[o + lane] = wi[lane];
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
                         const int j = lane + 32 * q;
@@ -839,39 +884,47 @@ __global__ void __launch_bounds__(256) chol_leaf128_kernel(float *A, long long l
         }
     }
     for (int ib = 1; ib < nb; ++ib) {
-        const int o = ib * 32, w = min(32, s - o), hw = (w + 1) >> 1;
+        const int o = ib * 32, w = min(32, s - o), hw = (w + 3) >> 2;
         for (int idx = warp; idx < ib * hw; idx += 8) {    // W[32 k + r][c] = sum_{q in [32 k, o)} L[o + r][q] X[q][32 k + c]
-            const int k = idx / hw, r0 = 2 * (idx - k * hw), r1 = r0 + 1;
-            const T *l0 = L + (o + r0) * ls, *l1 = L + (o + (r1 < w ? r1 : r0)) * ls;
-            T a0 = (T)0, a1 = (T)0;
+            const int k = idx / hw, r0 = 4 * (idx - k * hw);
+            const float *l[4];
+            float a[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) { l[t] = L + (o + min(r0 + t, w - 1)) * ls; a[t] = 0.f; }
+#pragma unroll 8
             for (int q = k * 32; q < o; ++q) {
-                const T xv = X[q * ls + k * 32 + lane];
-                a0 += l0[q] * xv;
-                a1 += l1[q] * xv;
+                const float xv = X[q * ls + k * 32 + lane];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) a[t] += l[t][q] * xv;
             }
-            W[(k * 32 + r0) * 33 + lane] = a0;
-            if (r1 < w) W[(k * 32 + r1) * 33 + lane] = a1;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (r0 + t < w) W[(k * 32 + r0 + t) * 33 + lane] = a[t];
         }
         __syncthreads();
         for (int idx = warp; idx < ib * hw; idx += 8) {    // X[o + r][32 k + c] = -sum_{q <= r} X_ii[r][q] W[32 k + q][c]
-            const int k = idx / hw, r0 = 2 * (idx - k * hw), r1 = r0 + 1;
-            const T *d0 = X + (o + r0) * ls + o, *d1 = X + (o + (r1 < w ? r1 : r0)) * ls + o;
-            T a0 = (T)0, a1 = (T)0;
-            for (int q = 0; q <= r0; ++q) {
-                const T wv = W[(k * 32 + q) * 33 + lane];
-                a0 += d0[q] * wv;
-                a1 += d1[q] * wv;
+            const int k = idx / hw, r0 = 4 * (idx - k * hw);
+            const float *d[4];
+            float a[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) { d[t] = X + (o + min(r0 + t, w - 1)) * ls + o; a[t] = 0.f; }
+            const int qn = min(r0 + 4, w);                 // (X_ii is zero above its diagonal)
+#pragma unroll 4
+            for (int q = 0; q < qn; ++q) {
+                const float wv = W[(k * 32 + q) * 33 + lane];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) a[t] += d[t][q] * wv;
             }
-            if (r1 < w) a1 += d1[r1] * W[(k * 32 + r1) * 33 + lane];
-            X[(o + r0) * ls + k * 32 + lane] = -a0;
-            if (r1 < w) X[(o + r1) * ls + k * 32 + lane] = -a1;
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (r0 + t < w) X[(o + r0 + t) * ls + k * 32 + lane] = -a[t];
         }
         __syncthreads();
     }
     for (int r = warp; r < s; r += 8)
         for (int c = lane; c < s; c += 32) {
-            A[(long long)r * lda + c] = (c <= r) ? L[r * ls + c] : (T)0;
-            Rinv[(long long)r * ldr + c] = (c <= r) ? X[r * ls + c] : (T)0;
+            A[(long long)r * lda + c] = (c <= r) ? L[r * ls + c] : 0.f;
+            Rinv[(long long)r * ldr + c] = (c <= r) ? X[r * ls + c] : 0.f;
         }
 }
 
@@ -879,7 +932,7 @@ __global__ void __launch_bounds__(256) chol_leaf128_kernel(float *A, long long l
 static size_t chol_leaf_smem(int s, bool fp64)
 {
     return fp64 ? (2 * (size_t)s * (s | 1) + 32 * 33 + 64) * sizeof(double)
-                : (2 * (size_t)s * (s + 1) + 34 * (size_t)s) * sizeof(float);
+                : (2 * (size_t)s * (s | 1) + 34 * (size_t)s) * sizeof(float);
 }
 
 template <class T>
