@@ -85,17 +85,49 @@ __device__ __forceinline__ unsigned long long smem_desc(uint32_t addr)
 constexpr uint32_t TC_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
                               ((uint32_t)(TC_BM >> 4) << 24);
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, unsigned long long a, unsigned long long b, uint32_t acc)
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, unsigned long long a, unsigned long long b, uint32_t acc,
+                                         uint32_t pred)
 {
     asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(TC_IDESC), "r"(acc));
+        "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(TC_IDESC), "r"(acc), "r"(pred));
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t bar)
+__device__ __forceinline__ void mma_commit_if(uint32_t bar, uint32_t pred)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+        "r"(pred)
+        : "memory");
+}
+
+// 1 in one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+    return e;
+}
+
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t *r)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+
+// waits for the loads in flight; r, which one of them fills, is not read before
+__device__ __forceinline__ void tmem_wait16(uint32_t *r)
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
 }
 
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_constant__ TcArgs g)
@@ -172,70 +204,87 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
         }
     } else if (warp == TC_MMA_WARP) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            bool ok = true;
-            for (int q = 0; q < nkb; ++q) {
-                const int s = q % TC_STAGES;
-                if (!mbar_wait(b_full + 8 * s, (uint32_t)((q / TC_STAGES) & 1), g.wait_limit)) { ok = false; break; }
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t st = smem_u32(smem + s * TC_STAGE_BYTES);
-                const uint32_t ah = st, al = st + TC_A_BYTES / 2;
-                const uint32_t bh = st + TC_A_BYTES, bl = st + TC_A_BYTES + TC_B_BYTES / 2;
+        // The warp runs converged and one elected lane issues: the operands stay in uniform
+        // registers, and six products of 128 clocks a stage are not held up by their issue.
+        const uint32_t leader = elect_one();
+        bool ok = true;
+        int s = 0;
+        uint32_t phase = 0;
+#pragma unroll 1
+        for (int q = 0; q < nkb; ++q) {
+            if (!mbar_wait(b_full + 8 * s, phase, g.wait_limit)) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t st = smem_u32(smem) + s * TC_STAGE_BYTES;
+            const uint32_t ah = st, al = st + TC_A_BYTES / 2;
+            const uint32_t bh = st + TC_A_BYTES, bl = st + TC_A_BYTES + TC_B_BYTES / 2;
 #pragma unroll
-                for (int kk = 0; kk < TC_BK / 8; ++kk) {           // K = 8 TF32 = 32 bytes per instruction
-                    const uint32_t off = kk * 32;
-                    mma_tf32(tmem, smem_desc(al + off), smem_desc(bh + off), (q > 0 || kk > 0) ? 1u : 0u);
-                    mma_tf32(tmem, smem_desc(ah + off), smem_desc(bl + off), 1u);
-                    mma_tf32(tmem, smem_desc(ah + off), smem_desc(bh + off), 1u);
-                }
-                mma_commit(b_empty + 8 * s);                   // stage s is free when these MMAs retire
+            for (int kk = 0; kk < TC_BK / 8; ++kk) {           // K = 8 TF32 = 32 bytes per instruction
+                const uint32_t off = kk * 32;
+                mma_tf32(tmem, smem_desc(al + off), smem_desc(bh + off), (q > 0 || kk > 0) ? 1u : 0u, leader);
+                mma_tf32(tmem, smem_desc(ah + off), smem_desc(bl + off), 1u, leader);
+                mma_tf32(tmem, smem_desc(ah + off), smem_desc(bh + off), 1u, leader);
             }
-            if (nkb > 0) {
-                if (ok) mma_commit(b_done);
-                else { s_abort = 1; atomicExch(g.err, 2); }
-            }
-            // Every MMA issued has retired before TMEM and the stages go away, whatever
-            // the other roles did (an epilogue warp that gave up no longer waits for them).
-            mma_commit(b_drain);
-            mbar_wait(b_drain, 0u, TC_WAIT_LIMIT);
+            mma_commit_if(b_empty + 8 * s, leader);            // stage s is free when these MMAs retire
+            if (++s == TC_STAGES) { s = 0; phase ^= 1; }
         }
+        if (nkb > 0) {
+            if (ok) mma_commit_if(b_done, leader);
+            else if (leader) { s_abort = 1; atomicExch(g.err, 2); }
+        }
+        // Every MMA issued has retired before TMEM and the stages go away, whatever
+        // the other roles did (an epilogue warp that gave up no longer waits for them).
+        mma_commit_if(b_drain, leader);
+        mbar_wait(b_drain, 0u, TC_WAIT_LIMIT);
     } else {
-        // ---------------- epilogue warps ----------------
-        const int quad = warp & 3, c0 = (warp >> 2) * TC_ECOLS;
+        // ---------------- epilogue warps: 32 rows, 128 columns in blocks of 32 ----------------
+        // A thread reads one row of the accumulator; the block goes through the ring (free:
+        // every product has retired) so that a store covers 128 bytes of one row instead of
+        // 4 bytes of 32 rows (the products of a 12288 split: 151 ms so, 129 through the ring).
+        const int quad = warp & 3, c0 = (warp >> 2) * TC_ECOLS, r0 = i0 + quad * 32;
         bool have = nkb > 0;
         if (have && !mbar_wait(b_done, 0u, g.wait_limit)) { have = false; atomicExch(g.err, 3); }
+        have = __all_sync(0xffffffffu, have);
         asm volatile("tcgen05.fence::after_thread_sync;");
-        const int i = i0 + quad * 32 + lane;
-        float *C = g.C + (long long)z * g.sC + (long long)i * g.ldc;
-        const float *Cin = g.Cin ? g.Cin + (long long)z * g.sCin + (long long)i * g.ldcin : nullptr;
-        {   // nkb == 0: the product is zero and C = beta Cin; a failed wait writes nothing
+        float *T = reinterpret_cast<float *>(smem) + warp * (32 * 33);
+        if (have || nkb == 0) {   // nkb == 0: the product is zero and C = beta Cin; a failed wait writes nothing
 #pragma unroll 1
-            for (int cc = 0; cc < TC_ECOLS; cc += 16) {
-                float v[16];
+            for (int cc = 0; cc < TC_ECOLS; cc += 32) {
+                const int jb = j0 + c0 + cc, j = jb + lane;
+                if (r0 >= g.m || jb >= g.n || (g.lowerC && jb > r0 + 31)) break;
                 if (have) {
-                    uint32_t r[16];
+                    uint32_t ra[16], rb[16];
                     const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(c0 + cc);
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                          "=r"(r[15])
-                        : "r"(taddr));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) v[q] = 0.f;
-                }
-                if (i < g.m && (have || nkb == 0)) {
+                    tmem_ld16_nowait(taddr, ra);
+                    tmem_ld16_nowait(taddr + 16, rb);
+                    tmem_wait16(ra);
+                    tmem_wait16(rb);
+                    __syncwarp();                              // the block before has been read
 #pragma unroll
                     for (int q = 0; q < 16; ++q) {
-                        const int j = j0 + c0 + cc + q;
-                        if (j >= g.n || (g.lowerC && j > i)) continue;
-                        float o = g.alpha * v[q];
-                        if (g.beta != 0.f) o += g.beta * Cin[j];
-                        C[j] = o;
+                        T[lane * 33 + q] = __uint_as_float(ra[q]);
+                        T[lane * 33 + 16 + q] = __uint_as_float(rb[q]);
+                    }
+                    __syncwarp();
+                }
+                float *C = g.C + (long long)z * g.sC + j;
+                const float *Cin = g.beta != 0.f ? g.Cin + (long long)z * g.sCin + j : nullptr;
+                constexpr int NB = 8;                          // rows in flight of beta Cin
+#pragma unroll 1
+                for (int p = 0; p < 32; p += NB) {
+                    float cv[NB];
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        const int row = r0 + p + u;
+                        const bool in = row < g.m && j < g.n && !(g.lowerC && j > row);
+                        cv[u] = Cin && in ? Cin[(long long)row * g.ldcin] : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        const int row = r0 + p + u;
+                        if (row >= g.m || j >= g.n || (g.lowerC && j > row)) continue;
+                        const float v = have ? T[(p + u) * 33 + lane] : 0.f;
+                        C[(long long)row * g.ldc] = Cin ? __fmaf_rn(g.alpha, v, __fmul_rn(g.beta, cv[u]))
+                                                        : __fmul_rn(g.alpha, v);
                     }
                 }
             }
