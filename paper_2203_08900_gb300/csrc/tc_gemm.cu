@@ -9,22 +9,29 @@
 // lo = x - hi; the product is accumulated in FP32 in tensor memory as
 //     A_lo B_hi + A_hi B_lo + A_hi B_hi      (3xTF32, ~FP32 accuracy).
 //
-// Kernel layout (one CTA of 10 warps per 128 x 256 output tile):
+// Kernel layout (one CTA of 10 warps per 128 x BN output tile, BN = 64, 128 or 256):
 //   * the split pass writes, for every (row tile, 16-term k block), the hi
 //     and lo parts as one contiguous block already in the 64-byte-swizzled
 //     order the MMA descriptors read (A: 2 x 128 rows x 64 bytes = 16 KB,
-//     B: 2 x 256 rows x 64 bytes = 32 KB);
+//     B: 2 x BN rows x 64 bytes);
 //   * warp 8 streams one k block per stage with two cp.async.bulk copies into
-//     a 4-stage ring of 48 KB with full/empty mbarriers;
+//     a ring of 96 KB (4, 3 or 2 stages) with full/empty mbarriers;
 //   * warp 9 issues per stage 2 (K = 8) x 3 tcgen05.mma kind::tf32 (M = 128,
-//     N = 256) into one FP32 accumulator of 256 TMEM columns and frees each
+//     N = BN) into one FP32 accumulator of BN TMEM columns and frees each
 //     stage with tcgen05.commit;
 //   * warps 0-7 wait for the final commit and write C (warp w: TMEM lanes
-//     32 (w % 4) .., i.e. tile rows, and columns 128 (w / 4) ..).
+//     32 (w % 4) .., i.e. tile rows, and columns BN/2 (w / 4) ..), through the
+//     ring: written from the accumulator's lanes a store touches 32 rows.
+// Two CTAs share an SM, so that one's epilogue and first copies run under the
+// other's products.  A large product is bound by shared memory, 96 bytes of
+// operand reads and 64 of copies for every 128 clocks of products at BN = 256.
 // Every pipeline mbarrier wait is bounded by the caller's limit: on timeout the
 // kernel sets *err, skips the remaining work, waits (under a fixed, longer
 // bound) for its own bulk copies and MMAs in flight, frees its TMEM and returns.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <climits>
 
 #include "mbar.cuh"
 #include "pssd_internal.h"
@@ -33,19 +40,18 @@ namespace pssd {
 
 namespace {
 
-constexpr int TC_BM = 128, TC_BN = 256, TC_BK = 16;    // BK in FP32 elements = 64 bytes per row
-constexpr int TC_STAGES = 4;
+constexpr int TC_BM = 128, TC_BN_MAX = 256, TC_BK = 16;   // BK in FP32 elements = 64 bytes per row
 constexpr int TC_A_BYTES = 2 * TC_BM * TC_BK * 4;      // hi + lo, 16 KB
-constexpr int TC_B_BYTES = 2 * TC_BN * TC_BK * 4;      // hi + lo, 32 KB
-constexpr int TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;
-constexpr int TC_SMEM_BYTES = TC_STAGES * TC_STAGE_BYTES + 1024 /* alignment */ + 256 /* barriers */;
+__host__ __device__ constexpr int tc_b_bytes(int bn) { return 2 * bn * TC_BK * 4; }
+__host__ __device__ constexpr int tc_smem_bytes(int bn, int stages)
+{
+    return stages * (TC_A_BYTES + tc_b_bytes(bn)) + 1024 /* alignment */ + 256 /* barriers */;
+}
 constexpr unsigned long long TC_WAIT_LIMIT = 1ull << 26;   // default pipeline bound and the drain bound
-constexpr int TC_EPI_WARPS = 8;                        // warp w: lanes 32 (w % 4) .., columns 128 (w / 4) ..
-constexpr int TC_ECOLS = TC_BN / (TC_EPI_WARPS / 4);
+constexpr int TC_EPI_WARPS = 8;                        // warp w: lanes 32 (w % 4) .., columns BN/2 (w / 4) ..
 constexpr int TC_PRODUCER_WARP = TC_EPI_WARPS, TC_MMA_WARP = TC_EPI_WARPS + 1;
 constexpr int TC_THREADS = 32 * (TC_EPI_WARPS + 2);
 constexpr int TC_GROUP_M = 8;                          // row blocks per group of the tile order
-constexpr int TC_TMEM_COLS = TC_BN;
 
 struct TcArgs {
     const float *a, *b;                        // tiled split operands (see the split kernel)
@@ -81,17 +87,19 @@ __device__ __forceinline__ unsigned long long smem_desc(uint32_t addr)
     return d;
 }
 
-// instruction descriptor: kind::tf32, D = F32, A = B = TF32, both K-major, M = 128, N = 256
-constexpr uint32_t TC_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
-                              ((uint32_t)(TC_BM >> 4) << 24);
+// instruction descriptor: kind::tf32, D = F32, A = B = TF32, both K-major, M = 128, N = bn
+__host__ __device__ constexpr uint32_t tc_idesc(int bn)
+{
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
+}
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, unsigned long long a, unsigned long long b, uint32_t acc,
-                                         uint32_t pred)
+__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, unsigned long long a, unsigned long long b,
+                                         uint32_t idesc, uint32_t acc, uint32_t pred)
 {
     asm volatile(
         "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
         "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(TC_IDESC), "r"(acc), "r"(pred));
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(pred));
 }
 
 __device__ __forceinline__ void mma_commit_if(uint32_t bar, uint32_t pred)
@@ -130,8 +138,13 @@ __device__ __forceinline__ void tmem_wait16(uint32_t *r)
                  : "memory");
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_constant__ TcArgs g)
+template <int BN, int STAGES, int CTAS>
+__global__ void __launch_bounds__(TC_THREADS, CTAS) tc_gemm_kernel(const __grid_constant__ TcArgs g)
 {
+    constexpr int TC_BN = BN, TC_STAGES = STAGES, TC_B_BYTES = tc_b_bytes(BN), TC_TMEM_COLS = BN;
+    constexpr int TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;
+    constexpr int TC_ECOLS = TC_BN / (TC_EPI_WARPS / 4);
+    static_assert(TC_EPI_WARPS * 32 * 33 * 4 <= TC_STAGES * TC_STAGE_BYTES, "the epilogue's blocks go into the ring");
     // grouped tile order: runs of TC_GROUP_M row blocks sweep the column blocks together
     const int mt = (g.m + TC_BM - 1) / TC_BM, nt = (g.n + TC_BN - 1) / TC_BN;
     const int pid = blockIdx.x, per_group = TC_GROUP_M * nt;
@@ -206,7 +219,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
         // ---------------- MMA issuer ----------------
         // The warp runs converged and one elected lane issues: the operands stay in uniform
         // registers, and six products of 128 clocks a stage are not held up by their issue.
-        const uint32_t leader = elect_one();
+        const uint32_t leader = elect_one(), idesc = tc_idesc(BN);
         bool ok = true;
         int s = 0;
         uint32_t phase = 0;
@@ -220,9 +233,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
 #pragma unroll
             for (int kk = 0; kk < TC_BK / 8; ++kk) {           // K = 8 TF32 = 32 bytes per instruction
                 const uint32_t off = kk * 32;
-                mma_tf32(tmem, smem_desc(al + off), smem_desc(bh + off), (q > 0 || kk > 0) ? 1u : 0u, leader);
-                mma_tf32(tmem, smem_desc(ah + off), smem_desc(bl + off), 1u, leader);
-                mma_tf32(tmem, smem_desc(ah + off), smem_desc(bh + off), 1u, leader);
+                mma_tf32(tmem, smem_desc(al + off), smem_desc(bh + off), idesc, (q > 0 || kk > 0) ? 1u : 0u, leader);
+                mma_tf32(tmem, smem_desc(ah + off), smem_desc(bl + off), idesc, 1u, leader);
+                mma_tf32(tmem, smem_desc(ah + off), smem_desc(bh + off), idesc, 1u, leader);
             }
             mma_commit_if(b_empty + 8 * s, leader);            // stage s is free when these MMAs retire
             if (++s == TC_STAGES) { s = 0; phase ^= 1; }
@@ -236,7 +249,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
         mma_commit_if(b_drain, leader);
         mbar_wait(b_drain, 0u, TC_WAIT_LIMIT);
     } else {
-        // ---------------- epilogue warps: 32 rows, 128 columns in blocks of 32 ----------------
+        // ---------------- epilogue warps: 32 rows, BN / 2 columns in blocks of 32 ----------------
         // A thread reads one row of the accumulator; the block goes through the ring (free:
         // every product has retired) so that a store covers 128 bytes of one row instead of
         // 4 bytes of 32 rows (the products of a 12288 split: 151 ms so, 129 through the ring).
@@ -331,6 +344,10 @@ __global__ void __launch_bounds__(256) tf32_split_kernel(TcOperand a, TcOperand 
     __shared__ float T[32][33];
     const int z = blockIdx.z;
     const int r0 = (isA ? (int)blockIdx.y : (int)blockIdx.y - nA) * 32, p0 = blockIdx.x * 32;
+    // A row tile's k range ends (begins) at the end (start) of its triangle: blocks beyond are never
+    // read (R^{-T} R^{-1}, 4 of order 1024: 36 us, 23 without them).
+    const int t0 = r0 / tile_rows * tile_rows;
+    if ((tri == TRI_LOWER && p0 >= t0 + tile_rows) || (tri == TRI_UPPER && p0 + 32 <= t0)) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8
     X += (long long)z * sb;
     // load the 32 x 32 block in the orientation that is contiguous in memory
@@ -378,15 +395,54 @@ __global__ void __launch_bounds__(256) tf32_split_kernel(TcOperand a, TcOperand 
 size_t tc_gemm_workspace_bytes(const GemmArgs &g)
 {
     const long long kp = (g.k + 15) / 16 * 16;
-    const long long mp = (g.m + TC_BM - 1) / TC_BM * TC_BM, np = (g.n + TC_BN - 1) / TC_BN * TC_BN;
+    const long long mp = (g.m + TC_BM - 1) / TC_BM * TC_BM, np = (g.n + TC_BN_MAX - 1) / TC_BN_MAX * TC_BN_MAX;
     return (size_t)(2 * (mp + np) * kp * g.batch) * sizeof(float) + 1024;
 }
 
 namespace {
-void tc_layout(const GemmArgs &g, void *ws, int &kp, int &mp, int &np, float *&ta, float *&tb)
+struct TcTile { int bn; int (*launch)(const TcArgs &, cudaStream_t); };
+
+template <int BN, int STAGES, int CTAS>
+int tc_launch_tile(const TcArgs &a, cudaStream_t s)
+{
+    const auto kernel = tc_gemm_kernel<BN, STAGES, CTAS>;
+    if (!ensure_dynamic_smem((const void *)kernel, tc_smem_bytes(BN, STAGES))) return -2;
+    const dim3 grid(((a.n + BN - 1) / BN) * ((a.m + TC_BM - 1) / TC_BM), 1, a.batch);
+    kernel<<<grid, TC_THREADS, tc_smem_bytes(BN, STAGES), s>>>(a); count_launch();
+    return 0;
+}
+
+// The tile width that takes the least time, counted in rounds of two CTAs an SM.  A CTA's round
+// costs 91 (64 columns), 128 or 241 (256) -- the measured times of k = 2048 products of many
+// rounds: 344, 276 and 263 us for 4 x 2048^3.  Wide tiles read A less often, narrow ones fill the
+// chip with a small product: 4 x 500^3 18, 24, 38 us (34 with one CTA an SM and four stages);
+// 4 x 1024^3 61, 47, 72; 6144^3 2006, 1458, 1366.  With a triangular operand the work differs from
+// tile to tile, there are no rounds, and 256 columns compute more of what is zero: 304 us with
+// 128, 351 with 256 for R^{-T} R^{-1} of order 6144.
+TcTile tc_tile(const GemmArgs &g)
+{
+    static const struct { TcTile tile; long long cost; } t[] = {
+        {{64, tc_launch_tile<64, 4, 2>}, 91}, {{128, tc_launch_tile<128, 3, 2>}, 128}, {{256, tc_launch_tile<256, 2, 2>}, 241}};
+    const long long slots = 2 * 152, mt = (g.m + TC_BM - 1) / TC_BM;
+    const bool tri = g.triA != TRI_NONE || g.triB != TRI_NONE;
+    TcTile best = t[0].tile;
+    long long least = LLONG_MAX;
+    for (const auto &x : t) {
+        if (tri && x.tile.bn == 256) break;
+        const long long nt = (g.n + x.tile.bn - 1) / x.tile.bn;
+        long long tiles = g.lowerC ? 0 : mt * nt;
+        for (long long i = 0; g.lowerC && i < mt; ++i)
+            tiles += std::min(nt, (i * TC_BM + TC_BM - 1) / x.tile.bn + 1);
+        const long long c = (tiles * g.batch + slots - 1) / slots * x.cost;
+        if (c < least) { least = c; best = x.tile; }
+    }
+    return best;
+}
+
+void tc_layout(const GemmArgs &g, void *ws, int bn, int &kp, int &mp, int &np, float *&ta, float *&tb)
 {
     kp = (g.k + 15) / 16 * 16;
-    mp = (g.m + TC_BM - 1) / TC_BM * TC_BM; np = (g.n + TC_BN - 1) / TC_BN * TC_BN;
+    mp = (g.m + TC_BM - 1) / TC_BM * TC_BM; np = (g.n + bn - 1) / bn * bn;
     float *base = (float *)(((uintptr_t)ws + 255) & ~(uintptr_t)255);
     ta = base; tb = ta + (size_t)2 * mp * kp * g.batch;
 }
@@ -396,12 +452,13 @@ void tc_layout(const GemmArgs &g, void *ws, int &kp, int &mp, int &np, float *&t
 int tc_gemm_prepare(const GemmArgs &g, void *ws, cudaStream_t s)
 {
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return 0;
+    const int bn = tc_tile(g).bn;
     int kp, mp, np; float *ta, *tb;
-    tc_layout(g, ws, kp, mp, np, ta, tb);
+    tc_layout(g, ws, bn, kp, mp, np, ta, tb);
     // A: rows i of op(A); B: rows j of op(B)^T (op(B)[p][j] = B[p][j] or B[j][p]); both K-major
     const int triB = g.triB == TRI_LOWER ? TRI_UPPER : (g.triB == TRI_UPPER ? TRI_LOWER : TRI_NONE);
     const TcOperand oa{(const float *)g.A, g.lda, g.sA, g.ta, g.m, mp, TC_BM, g.triA, (const float *)g.kscale, ta};
-    const TcOperand ob{(const float *)g.B, g.ldb, g.sB, g.tb ? 0 : 1, g.n, np, TC_BN, triB, nullptr, tb};
+    const TcOperand ob{(const float *)g.B, g.ldb, g.sB, g.tb ? 0 : 1, g.n, np, bn, triB, nullptr, tb};
     const int nA = mp / 32, nB = np / 32;
     tf32_split_kernel<<<dim3((kp + 31) / 32, nA + nB, g.batch), 256, 0, s>>>(oa, ob, g.k, kp, nA); count_launch();
     return 0;
@@ -411,9 +468,9 @@ int tc_gemm_prepare(const GemmArgs &g, void *ws, cudaStream_t s)
 int tc_gemm_run(const GemmArgs &g, void *ws, int *err, cudaStream_t s)
 {
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return 0;
-    if (!ensure_dynamic_smem((const void *)tc_gemm_kernel, TC_SMEM_BYTES)) return -2;
+    const TcTile t = tc_tile(g);
     int kp, mp, np; float *ta, *tb;
-    tc_layout(g, ws, kp, mp, np, ta, tb);
+    tc_layout(g, ws, t.bn, kp, mp, np, ta, tb);
     TcArgs a;
     a.a = ta; a.b = tb; a.kblocks = kp / 16;
     a.m = g.m; a.n = g.n; a.k = g.k; a.batch = g.batch; a.m_pad = mp; a.n_pad = np;
@@ -423,9 +480,7 @@ int tc_gemm_run(const GemmArgs &g, void *ws, int *err, cudaStream_t s)
     a.alpha = (float)g.alpha; a.beta = (float)g.beta;
     a.err = err;
     a.wait_limit = g.wait_limit > 0 ? (unsigned long long)g.wait_limit : TC_WAIT_LIMIT;
-    dim3 grid(((g.n + TC_BN - 1) / TC_BN) * ((g.m + TC_BM - 1) / TC_BM), 1, g.batch);
-    tc_gemm_kernel<<<grid, TC_THREADS, TC_SMEM_BYTES, s>>>(a); count_launch();
-    return 0;
+    return t.launch(a, s);
 }
 
 // ws: device workspace of tc_gemm_workspace_bytes(g) bytes; err: device int (0 on entry)
