@@ -274,28 +274,42 @@ constexpr int GM_DOUBLE = -1;
 
 template <class T> int gm_of() { return std::is_same<T, float>::value ? GM_F32 : GM_DOUBLE; }
 
-void gemm(pssd_handle h, const GemmArgs &g0)
+// the engine that takes a product
+int gemm_mode(pssd_handle h, const GemmArgs &g)
 {
-    if (g0.m <= 0 || g0.n <= 0 || g0.batch <= 0) return;
-    GemmArgs g = g0;
-    if (g.mode < 0) g.mode = h->dmode;
-    g.wait_limit = h->wait_limit;
-    double fl = h->prof ? 2.0 * gemm_macs(g) : 0.0;
-    Mark mk = mark(h);
-    if (g.mode == GM_OZ && !h->derr) g.mode = GM_DF;   // (no error flag outside a guarded call)
+    int mode = g.mode < 0 ? h->dmode : g.mode;
+    if (mode == GM_OZ && !h->derr) mode = GM_DF;   // (no error flag outside a guarded call)
     // Small products: the slice engine's two launches and its tile latency dominate, and the
     // FP64 pipes finish first (64^3: 3 us against 14 us; 192^3: 16 against 24; 256^3: 35 against
     // 27; the estimates decide).  Upstream of the mixed mode's FP32 iteration the
     // engines are pinned -- float pairs for thin or tiny products, slices for the rest: the
     // iteration turns a flipped last bit of its input into a change of the size of its own
     // error, so mixed results would otherwise move with every choice made here.
-    if (g.mode == GM_OZ && !h->force_engine) {
+    if (mode == GM_OZ && !h->force_engine) {
         if (h->pinned) {
-            if (g.k < 16 || (double)g.m * g.n * g.k * g.batch < 262144.0) g.mode = GM_DF;
+            if (g.k < 16 || (double)g.m * g.n * g.k * g.batch < 262144.0) mode = GM_DF;
         } else if (dgemm_time_us(g) <= oz_gemm_time_us(g)) {
-            g.mode = GM_F64;
+            mode = GM_F64;
         }
     }
+    return mode;
+}
+
+// whether a product's engine works on its own copy of op(A) and op(B), so that C may be one of them
+bool gemm_copies(pssd_handle h, const GemmArgs &g)
+{
+    const int mode = gemm_mode(h, g);
+    return mode == GM_OZ || mode == GM_DF || (mode == GM_F32 && h->use_tc && h->derr);
+}
+
+void gemm(pssd_handle h, const GemmArgs &g0)
+{
+    if (g0.m <= 0 || g0.n <= 0 || g0.batch <= 0) return;
+    GemmArgs g = g0;
+    g.mode = gemm_mode(h, g0);
+    g.wait_limit = h->wait_limit;
+    double fl = h->prof ? 2.0 * gemm_macs(g) : 0.0;
+    Mark mk = mark(h);
     if (g.mode == GM_DF) {
         // split each FP64 operand into compact float pairs once (stream-ordered temporaries)
         const int ra = g.ta ? g.k : g.m, cla = g.ta ? g.m : g.k;
@@ -411,14 +425,18 @@ void chol_rec(pssd_handle h, T *A, int off, int s, long long lda, long long sA, 
     chol_rec<T>(h, A, off, hh, lda, sA, batch, Rinv, sR, dinfo, tmp, sT);
     T *A21 = A + (long long)(off + hh) * lda + off;
     T *A22 = A + (long long)(off + hh) * lda + (off + hh);
-    {   // L21 = A21 L11^{-T} into tmp (the product reads whole rows of A21), then back
+    {   // L21 = A21 L11^{-T}: in place where the engine has copied A21, else into tmp and back
+        // (the product reads whole rows of A21: a pass, 9.1 instead of 9.3 ms of an n=1000 mixed sign)
         GemmArgs g; g.mode = gm_of<T>(); g.m = q; g.n = hh; g.k = hh; g.batch = batch;
         g.A = A21; g.lda = lda; g.sA = sA;
         g.B = Rinv + (long long)off * lda + off; g.ldb = lda; g.sB = sR; g.tb = 1; g.triB = TRI_UPPER;
-        g.C = tmp; g.ldc = hh; g.sC = sT;
+        const bool in_place = gemm_copies(h, g);
+        g.C = in_place ? A21 : tmp; g.ldc = in_place ? lda : hh; g.sC = in_place ? sA : sT;
         gemm(h, g);
-        Timed t(h, K_HBM, 0, 2.0 * sizeof(T) * q * (double)hh * batch);
-        copy_batched<T>(tmp, hh, sT, A21, lda, sA, q, hh, batch, h->stream);
+        if (!in_place) {
+            Timed t(h, K_HBM, 0, 2.0 * sizeof(T) * q * (double)hh * batch);
+            copy_batched<T>(tmp, hh, sT, A21, lda, sA, q, hh, batch, h->stream);
+        }
     }
     {   // A22 -= L21 L21^T (lower)
         GemmArgs g; g.mode = gm_of<T>(); g.m = q; g.n = q; g.k = hh; g.batch = batch;
