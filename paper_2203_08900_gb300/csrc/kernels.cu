@@ -52,7 +52,7 @@ bool ensure_dynamic_smem(const void *func, int bytes)
 //           so the FP64 pipe -- 1/64 of the FP32 rate on GB300 -- only sees
 //           the flushes.  Relative error per 128-term block ~2^-46.
 // --------------------------------------------------------------------------
-constexpr int GBM = 64, GBN = 64, GBK = 16;
+constexpr int GBK = 16;                              // tile of Q x Q outputs a thread, 16 x 16 threads
 
 template <class T>
 __device__ __forceinline__ T load_op(const T *P, long long ld, int trans, int r, int c)
@@ -60,10 +60,11 @@ __device__ __forceinline__ T load_op(const T *P, long long ld, int trans, int r,
     return trans ? P[(long long)c * ld + r] : P[(long long)r * ld + c];
 }
 
-template <int MODE>
+template <int MODE, int Q>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
 {
     using T = typename std::conditional<MODE == GM_F32, float, double>::type;
+    constexpr int GBM = 16 * Q, GBN = 16 * Q;
     const int z = blockIdx.z;
     const int i0 = blockIdx.y * GBM, j0 = blockIdx.x * GBN;
     if (i0 >= g.m || j0 >= g.n) return;
@@ -86,20 +87,20 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
     __shared__ float Asl[MODE == GM_DF ? GBK : 1][GBM + 1], Bsl[MODE == GM_DF ? GBK : 1][GBN + 1];
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
-    float ah_[4][4], al_[4][4];   // DF running float pair (unused otherwise)
+    T acc[Q][Q];
+    float ah_[Q][Q], al_[Q][Q];   // DF running float pair (unused otherwise)
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < Q; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) { acc[a][b] = 0; ah_[a][b] = 0.f; al_[a][b] = 0.f; }
+        for (int b = 0; b < Q; ++b) { acc[a][b] = 0; ah_[a][b] = 0.f; al_[a][b] = 0.f; }
 
     int kt_count = 0;
     for (int kt = kbeg; kt < kend; kt += GBK) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < Q; ++u) {
             int e = tid + 256 * u;
             int il, pl;
-            if (g.ta == 0) { il = e >> 4; pl = e & 15; } else { pl = e >> 6; il = e & 63; }
+            if (g.ta == 0) { il = e >> 4; pl = e & 15; } else { pl = e / GBM; il = e % GBM; }
             int i = i0 + il, p = kt + pl;
             bool ok = (i < g.m) && (p < kend);
             if (g.triA == TRI_LOWER) ok = ok && (p <= i);
@@ -122,10 +123,10 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < Q; ++u) {
             int e = tid + 256 * u;
             int jl, pl;
-            if (g.tb == 0) { pl = e >> 6; jl = e & 63; } else { jl = e >> 4; pl = e & 15; }
+            if (g.tb == 0) { pl = e / GBN; jl = e % GBN; } else { jl = e >> 4; pl = e & 15; }
             int j = j0 + jl, p = kt + pl;
             bool ok = (j < g.n) && (p < kend);
             if (g.triB == TRI_LOWER) ok = ok && (p >= j);
@@ -145,27 +146,27 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
         if (MODE != GM_DF) {
 #pragma unroll
             for (int p = 0; p < GBK; ++p) {
-                S a[4], b[4];
+                S a[Q], b[Q];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { a[q] = As[p][ty + 16 * q]; b[q] = Bs[p][tx + 16 * q]; }
+                for (int q = 0; q < Q; ++q) { a[q] = As[p][ty + 16 * q]; b[q] = Bs[p][tx + 16 * q]; }
 #pragma unroll
-                for (int qa = 0; qa < 4; ++qa)
+                for (int qa = 0; qa < Q; ++qa)
 #pragma unroll
-                    for (int qb = 0; qb < 4; ++qb) acc[qa][qb] = fma((T)a[qa], (T)b[qb], acc[qa][qb]);
+                    for (int qb = 0; qb < Q; ++qb) acc[qa][qb] = fma((T)a[qa], (T)b[qb], acc[qa][qb]);
             }
         } else {
 #pragma unroll 4
             for (int p = 0; p < GBK; ++p) {
-                float ahv[4], alv[4], bhv[4], blv[4];
+                float ahv[Q], alv[Q], bhv[Q], blv[Q];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < Q; ++q) {
                     ahv[q] = As[p][ty + 16 * q]; alv[q] = Asl[p][ty + 16 * q];
                     bhv[q] = Bs[p][tx + 16 * q]; blv[q] = Bsl[p][tx + 16 * q];
                 }
 #pragma unroll
-                for (int qa = 0; qa < 4; ++qa)
+                for (int qa = 0; qa < Q; ++qa)
 #pragma unroll
-                    for (int qb = 0; qb < 4; ++qb) {
+                    for (int qb = 0; qb < Q; ++qb) {
                         // rounded intrinsics: never contracted, so the transformations stay error-free
                         float ph = __fmul_rn(ahv[qa], bhv[qb]);
                         float pe = __fmaf_rn(ahv[qa], bhv[qb], -ph);                 // hi*hi = ph + pe exactly
@@ -180,9 +181,9 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
             }
             if (((++kt_count) & 7) == 0) {   // flush the float pairs into FP64 every 128 k
 #pragma unroll
-                for (int qa = 0; qa < 4; ++qa)
+                for (int qa = 0; qa < Q; ++qa)
 #pragma unroll
-                    for (int qb = 0; qb < 4; ++qb) {
+                    for (int qb = 0; qb < Q; ++qb) {
                         acc[qa][qb] += (double)ah_[qa][qb] + (double)al_[qa][qb];
                         ah_[qa][qb] = 0.f; al_[qa][qb] = 0.f;
                     }
@@ -192,20 +193,20 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g)
     }
     if (MODE == GM_DF) {
 #pragma unroll
-        for (int qa = 0; qa < 4; ++qa)
+        for (int qa = 0; qa < Q; ++qa)
 #pragma unroll
-            for (int qb = 0; qb < 4; ++qb) acc[qa][qb] += (double)ah_[qa][qb] + (double)al_[qa][qb];
+            for (int qb = 0; qb < Q; ++qb) acc[qa][qb] += (double)ah_[qa][qb] + (double)al_[qa][qb];
     }
 
     T *C = (T *)g.C + (long long)z * g.sC;
     const T *Cin = g.Cin ? (const T *)g.Cin + (long long)z * g.sCin : nullptr;
     const T alpha = (T)g.alpha, beta = (T)g.beta;
 #pragma unroll
-    for (int qa = 0; qa < 4; ++qa) {
+    for (int qa = 0; qa < Q; ++qa) {
         int i = i0 + ty + 16 * qa;
         if (i >= g.m) continue;
 #pragma unroll
-        for (int qb = 0; qb < 4; ++qb) {
+        for (int qb = 0; qb < Q; ++qb) {
             int j = j0 + tx + 16 * qb;
             if (j >= g.n) continue;
             if (g.lowerC && j > i) continue;
@@ -409,10 +410,21 @@ static void dgemm_launch(const GemmArgs &g, cudaStream_t s)
 void gemm_launch(const GemmArgs &g, cudaStream_t s)
 {
     if (g.m <= 0 || g.n <= 0 || g.batch <= 0) return;
-    dim3 grid((g.n + GBN - 1) / GBN, (g.m + GBM - 1) / GBM, g.batch);
+    const auto grid = [&](int tile) { return dim3((g.n + tile - 1) / tile, (g.m + tile - 1) / tile, g.batch); };
+    const dim3 g64 = grid(64);
     switch (g.mode) {
-    case GM_F32: gemm_kernel<GM_F32><<<grid, 256, 0, s>>>(g); count_launch(); break;
-    case GM_DF: gemm_kernel<GM_DF><<<grid, 256, 0, s>>>(g); count_launch(); break;
+    case GM_F32: gemm_kernel<GM_F32, 4><<<g64, 256, 0, s>>>(g); count_launch(); break;
+    case GM_DF:
+        // A float-pair multiply-add is 13 instructions, so a small product takes as long as a thread's
+        // share of it: tiles of 16 while they fit on the chip (32 x 64 x 64: 22 us, 2 us with them).
+        // Up to k = 128, where no flush lies inside the product, a tile's k range does not show in the
+        // result's bits.
+        if (g.k <= 128 && 16ll * g64.x * g64.y * g64.z <= 4 * 152)
+            gemm_kernel<GM_DF, 1><<<grid(16), 256, 0, s>>>(g);
+        else
+            gemm_kernel<GM_DF, 4><<<g64, 256, 0, s>>>(g);
+        count_launch();
+        break;
     default: dgemm_launch(g, s); break;
     }
 }
