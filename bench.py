@@ -638,7 +638,7 @@ def main():
     return 0
 
 
-KERNEL_NAMES = {"dgemm": "gemm_kernel<GM_F64> (FP64 DFMA, 64x64x16 tiles)",
+KERNEL_NAMES = {"dgemm": "dgemm_kernel<32|16|8> (FP64 DFMA)",
                 "sgemm": "gemm_kernel<GM_F32> (FP32 FFMA)",
                 "dfgemm": "gemm_kernel<GM_DF> (FP64 emulated with float pairs on the FP32 pipe)",
                 "tcgemm": "tc_gemm_kernel (tcgen05 kind::tf32, 3xTF32)",
