@@ -1616,14 +1616,27 @@ void give_back_helper(pssd_handle_s *x)
     x->root->idle_helpers.push_back(x);
 }
 
+// memory that helpers at rest hold
+void free_idle_helpers(pssd_handle h)
+{
+    pssd_handle_s *root = h->root ? h->root : h;
+    std::lock_guard<std::mutex> lk(root->helper_mu);
+    for (auto *x : root->idle_helpers) {
+        cudaStreamSynchronize(x->stream);
+        for (auto &c : x->chunks) if (c.owned) cudaFree(c.base);
+        x->chunks.clear();
+    }
+}
+
 // The two halves of a division are independent, and below order 1000 or so neither fills the
 // GPU: a node is a chain of small launches and host reads.  The second half runs in a thread of
 // its own on a helper's stream while there is a helper (so up to four chains at a time), with
 // the same seeds and operations as one after the other.  casida_eig at k = 1024: 103 -> 70 ms,
-// zeig at n = 400: 76 -> 44 ms.
+// zeig at n = 400: 76 -> 44 ms.  A half that finds no memory beside the other runs after it.
 int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, int depth, int *maxdepth)
 {
     int da = *maxdepth, db = *maxdepth;
+    const Mark before = mark(h);
     pssd_handle_s *x = std::min(a.m, b.m) > leaf ? acquire_helper(h) : nullptr;
     std::thread second;
     cudaEvent_t done = nullptr;
@@ -1673,6 +1686,9 @@ int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, in
     std::exception_ptr thrown;
     try {
         st_a = sym_eig_node(h, a.B, a.m, a.W, a.w, leaf, depth, &da, a.seed);
+    } catch (Fail &f) {
+        if (f.code == PSSD_ERR_ALLOC) st_a = f.code;
+        else thrown = std::current_exception();
     } catch (...) {
         thrown = std::current_exception();
     }
@@ -1687,6 +1703,17 @@ int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, in
     if (thrown || st_a) cudaStreamSynchronize(x->stream);
     give_back_helper(x);
     if (thrown) std::rethrow_exception(thrown);
+    const bool short_a = st_a == PSSD_ERR_ALLOC, short_b = st_b == PSSD_ERR_ALLOC;
+    if ((short_a || short_b) && (short_a || !st_a) && (short_b || !st_b)) {
+        if (short_a) {
+            if (h->side) cudaStreamSynchronize(h->side);
+            cudaStreamSynchronize(h->stream);
+            release(h, before);
+        }
+        free_idle_helpers(h);
+        st_a = short_a ? sym_eig_node(h, a.B, a.m, a.W, a.w, leaf, depth, &da, a.seed) : PSSD_OK;
+        st_b = !st_a && short_b ? sym_eig_node(h, b.B, b.m, b.W, b.w, leaf, depth, &db, b.seed) : PSSD_OK;
+    }
     if (st_a || st_b) return st_a ? st_a : st_b;
     cuda_check(h, cudaStreamWaitEvent(h->stream, done, 0), "cudaStreamWaitEvent");
     *maxdepth = std::max(da, db);
