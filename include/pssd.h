@@ -486,7 +486,7 @@ int pssd_gsplit(pssd_handle h, int n, const signed char *sigma, const double *H,
  * = beta_j (device, 2 steps + 2 doubles).  power > 0: that many normalised power
  * steps from the Gaussian vector of seed 0x5eed, then out[0] = v^T op(A) v.
  * fused = 0: one launch per vector operation; fused = 1: the whole loop in one
- * thread-block-cluster launch (m <= 1024).  v0 (device, m, or NULL) receives the
+ * cooperative launch (m <= 1024).  v0 (device, m, or NULL) receives the
  * starting vector before normalisation.  Returns 0 or a negative argument index
  * (-6: power outside [0, 1000], or power = 0 with steps outside [1, m]). */
 #define PSSD_KRYLOV_SYM 0

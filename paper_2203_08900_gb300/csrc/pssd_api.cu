@@ -3832,7 +3832,7 @@ extern "C" int pssd_gsplit(pssd_handle h, int n, const signed char *sigma, const
 
 // ---------------------------------------------------------------------------
 // test hook: the Krylov loops behind the bounds, the shift search and the shift
-// screening, step by step or in one cluster launch, on the operators they use
+// screening, step by step or in one cooperative launch, on the operators they use
 // ---------------------------------------------------------------------------
 extern "C" int pssd_test_krylov(pssd_handle h, int op, int m, const double *A, int lda, int steps, int power,
                                 unsigned long long seed, int fused, double *out, double *v0)
