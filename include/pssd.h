@@ -504,6 +504,15 @@ int pssd_test_krylov(pssd_handle h, int op, int m, const double *A, int lda, int
 int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W, int ldw, double *w,
                       const pssd_opts *opts, pssd_info *info);
 
+/* Test hook: failures that a test makes on the host, without a GPU fault.  Sets a failure of
+ * the handle's later calls; value 0 takes it back (the default).  Returns 0, -2 (what) or -3
+ * (value < 0).
+ *   PSSD_FAULT_LAUNCH  1: in the symmetric recursion, the thread of a division's second half
+ *                      issues a launch that the runtime refuses */
+#define PSSD_FAULT_LAUNCH 0
+#define PSSD_FAULT_COUNT 1
+int pssd_test_fault(pssd_handle h, int what, long long value);
+
 /* ---------------------------------------------------------------------------
  * Profiling hooks (no counterpart in the paper; for measurement only).
  * With profiling on, each library kernel region on the handle's stream is

@@ -30,6 +30,7 @@ FLAG_EMU_SIMT = 4
 FLAG_NO_REFINE = 8
 FLAG_RECOMPUTE = 16
 METHOD_ZOLO, METHOD_DWH, METHOD_NEWTON = 0, 1, 2
+FAULT_LAUNCH = 0
 
 
 class Opts(ctypes.Structure):
@@ -72,7 +73,7 @@ EXPORTS = ["pssd_opts_init", "pssd_create", "pssd_destroy", "pssd_set_stream", "
            "pssd_test_gemm_f64", "pssd_workspace_bytes", "pssd_set_workspace", "pssd_workspace_peak",
            "pssd_device_alloc_count", "pssd_casida_sign", "pssd_casida_split", "pssd_casida_eig",
            "pssd_test_sym_eig", "pssd_sign_vjp_rev", "pssd_zsign", "pssd_zeig", "pssd_launch_count_phases",
-           "pssd_test_krylov", "pssd_gsign", "pssd_gsplit"]
+           "pssd_test_krylov", "pssd_gsign", "pssd_gsplit", "pssd_test_fault"]
 NOALLOC_MAX_N = 128
 MAX_N = 65535                 # PSSD_MAX_N: largest supported order
 
@@ -135,6 +136,7 @@ def lib():
     L.pssd_launch_count_phases.argtypes = [vp, ctypes.c_int]
     L.pssd_test_krylov.argtypes = [vp, ctypes.c_int, ctypes.c_int, vp, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                    ctypes.c_ulonglong, ctypes.c_int, vp, vp]
+    L.pssd_test_fault.argtypes = [vp, ctypes.c_int, ll]
     L.pssd_workspace_bytes.argtypes = [vp, ctypes.c_int, ctypes.POINTER(Opts), ctypes.POINTER(ctypes.c_size_t)]
     L.pssd_set_workspace.argtypes = [vp, vp, ctypes.c_size_t]
     L.pssd_workspace_peak.argtypes = [vp, ctypes.POINTER(ctypes.c_size_t)]
@@ -242,6 +244,10 @@ class Handle:
         b = ctypes.c_size_t(0)
         self._check(lib().pssd_workspace_peak(self._h, ctypes.byref(b)))
         return int(b.value)
+
+    def test_fault(self, what: int, value: int):
+        """Test hook: pssd_test_fault (FAULT_*; value 0 takes the failure back)."""
+        self._check(lib().pssd_test_fault(self._h, int(what), int(value)))
 
     def _check(self, st):
         if st:

@@ -83,6 +83,7 @@ struct pssd_handle_s {
     std::vector<cudaEvent_t> leaf_pending;     // leaves launched on `side` that the main stream has not joined
     std::vector<cudaEvent_t> sync_events;      // events without timing for the joins (pooled)
     size_t sync_used = 0;
+    long long fault[PSSD_FAULT_COUNT] = {0};   // pssd_test_fault (of the calling handle, root)
 };
 
 namespace {
@@ -91,6 +92,8 @@ namespace {
 // errors
 // ---------------------------------------------------------------------------
 struct Fail { int code; };
+
+pssd_handle_s *root_of(pssd_handle h) { return h->root ? h->root : h; }
 
 inline void cuda_check(pssd_handle h, cudaError_t e, const char *what)
 {
@@ -1586,10 +1589,14 @@ int sym_eig(pssd_handle h, const double *B, int m, double *W, double *w, int lea
 
 constexpr int MAX_HELPERS = 3;
 
+// a launch that the runtime refuses (no such block size), for pssd_test_fault
+__global__ void refused_kernel() {}
+void refused_launch(cudaStream_t s) { refused_kernel<<<1, 4096, 0, s>>>(); }
+
 // an idle helper of h's calling handle, or null: none left, or workspace that may not grow
 pssd_handle_s *acquire_helper(pssd_handle h)
 {
-    pssd_handle_s *root = h->root ? h->root : h;
+    pssd_handle_s *root = root_of(h);
     if (root->sequential || root->user_ws) return nullptr;
     std::lock_guard<std::mutex> lk(root->helper_mu);
     if (!root->idle_helpers.empty()) {
@@ -1619,7 +1626,7 @@ void give_back_helper(pssd_handle_s *x)
 // memory that helpers at rest hold
 void free_idle_helpers(pssd_handle h)
 {
-    pssd_handle_s *root = h->root ? h->root : h;
+    pssd_handle_s *root = root_of(h);
     std::lock_guard<std::mutex> lk(root->helper_mu);
     for (auto *x : root->idle_helpers) {
         cudaStreamSynchronize(x->stream);
@@ -1653,6 +1660,7 @@ int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, in
             second = std::thread([&, dev, ready, done]() {
                 cudaSetDevice(dev);
                 Mark mk = mark(x);
+                if (x->root->fault[PSSD_FAULT_LAUNCH]) refused_launch(x->stream);
                 try {
                     cuda_check(x, cudaStreamWaitEvent(x->stream, ready, 0), "cudaStreamWaitEvent");
                     st_b = sym_eig_node(x, b.B, b.m, b.W, b.w, leaf, depth, &db, b.seed);
@@ -1662,6 +1670,13 @@ int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, in
                     st_b = f.code;
                 } catch (...) {
                     st_b = PSSD_ERR_ALLOC;
+                }
+                // Launches are not checked one by one, and the runtime keeps their errors per
+                // thread: the check at the end of the call does not see this thread's.
+                const cudaError_t e = cudaGetLastError();
+                if (e != cudaSuccess) {
+                    x->last_err = std::string("kernel launch: ") + cudaGetErrorString(e);
+                    st_b = PSSD_ERR_CUDA;
                 }
                 if (st_b) {   // nothing of this half may still run when its operands go away
                     if (x->side) cudaStreamSynchronize(x->side);
@@ -3828,6 +3843,18 @@ extern "C" int pssd_gsplit(pssd_handle h, int n, const signed char *sigma, const
         cuda_check(h, cudaStreamSynchronize(h->stream), "sync");          // shat goes out of scope
         return PSSD_OK;
     });
+}
+
+// ---------------------------------------------------------------------------
+// test hook: host-made failures
+// ---------------------------------------------------------------------------
+extern "C" int pssd_test_fault(pssd_handle h, int what, long long value)
+{
+    if (!h) return -1;
+    if (what < 0 || what >= PSSD_FAULT_COUNT) return -2;
+    if (value < 0) return -3;
+    h->fault[what] = value;
+    return PSSD_OK;
 }
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,39 @@
+"""The two halves of a division side by side when something fails on the host (pssd_test_fault): what the second
+half's thread meets is reported as it would be on the calling thread, and the handle stays usable."""
+import pytest
+import torch
+
+import casida_inputs as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    from paper_2203_08900_gb300 import build as b
+    b.build()
+    import paper_2203_08900_gb300 as P
+    P.lib()
+    return P
+
+
+def _H(k, seed=11):
+    return torch.from_numpy(G.casida(k, ("uniform", 1.0, 10.0), seed=seed)[0]).cuda()
+
+
+@pytest.mark.parametrize("call", ["eig", "casida_eig"])
+def test_refused_launch_in_the_second_half_is_reported(P, call):
+    H = _H(200)
+    k = H.shape[0] // 2
+    blocks = H[:k, :k].contiguous(), H[:k, k:].contiguous()
+    h = P.Handle()
+    run = lambda: P.eig(H, handle=h) if call == "eig" else P.casida_eig(*blocks, handle=h)   # noqa: E731
+    D, V, _ = run()
+    h.test_fault(P.FAULT_LAUNCH, 1)
+    with pytest.raises(P.PssdError) as e:
+        run()
+    assert e.value.status == 6 and "kernel launch" in str(e.value)
+    h.test_fault(P.FAULT_LAUNCH, 0)
+    D1, V1, _ = run()
+    assert torch.equal(D1, D) and torch.equal(V1, V)
+    h.close()
