@@ -507,10 +507,16 @@ int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W,
 /* Test hook: failures that a test makes on the host, without a GPU fault.  Sets a failure of
  * the handle's later calls; value 0 takes it back (the default).  Returns 0, -2 (what) or -3
  * (value < 0).
- *   PSSD_FAULT_LAUNCH  1: in the symmetric recursion, the thread of a division's second half
- *                      issues a launch that the runtime refuses */
+ *   PSSD_FAULT_LAUNCH  in the symmetric recursion, a launch that the runtime refuses is issued by
+ *                      1: the thread of a division's second half, 2: the calling thread before it
+ *                      looks for a helper, 3: both
+ *   PSSD_FAULT_MEMORY  bytes that the workspaces of the handle and of its helpers may take
+ *                      together: an allocation beyond is refused by the runtime
+ *   PSSD_FAULT_STREAM  1: the runtime refuses the streams of new helpers */
 #define PSSD_FAULT_LAUNCH 0
-#define PSSD_FAULT_COUNT 1
+#define PSSD_FAULT_MEMORY 1
+#define PSSD_FAULT_STREAM 2
+#define PSSD_FAULT_COUNT 3
 int pssd_test_fault(pssd_handle h, int what, long long value);
 
 /* ---------------------------------------------------------------------------

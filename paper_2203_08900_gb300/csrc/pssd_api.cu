@@ -84,6 +84,7 @@ struct pssd_handle_s {
     std::vector<cudaEvent_t> sync_events;      // events without timing for the joins (pooled)
     size_t sync_used = 0;
     long long fault[PSSD_FAULT_COUNT] = {0};   // pssd_test_fault (of the calling handle, root)
+    std::atomic<long long> held{0};            // bytes of workspace allocated by it and its helpers (root)
 };
 
 namespace {
@@ -126,6 +127,28 @@ void release(pssd_handle h, Mark m)
     h->depth = m.depth;
 }
 
+// the handle's own chunks
+void free_chunks(pssd_handle h)
+{
+    for (auto &c : h->chunks)
+        if (c.owned) {
+            cudaFree(c.base);
+            root_of(h)->held -= (long long)c.cap;
+        }
+    h->chunks.clear();
+}
+
+// A launch refused earlier in the call, which the check at its end reports, before a call whose
+// failure is dealt with here: the runtime keeps one error per thread, the latest.
+struct PendingError {
+    cudaError_t e = cudaPeekAtLastError();
+    void clear_later(pssd_handle h) const
+    {
+        (void)cudaGetLastError();
+        cuda_check(h, e, "kernel launch");
+    }
+};
+
 void *walloc(pssd_handle h, size_t bytes)
 {
     bytes = (bytes + 255) & ~size_t(255);
@@ -153,9 +176,13 @@ void *walloc(pssd_handle h, size_t bytes)
     size_t cap = std::max(bytes, h->chunk_bytes);
     void *p = nullptr;
     g_device_allocs.fetch_add(1, std::memory_order_relaxed);
-    cudaError_t e = cudaMalloc(&p, cap);
+    const PendingError pending;
+    pssd_handle_s *root = root_of(h);
+    const long long limit = root->fault[PSSD_FAULT_MEMORY], held = root->held += (long long)cap;
+    cudaError_t e = cudaMalloc(&p, limit && held > limit ? size_t(1) << 60 : cap);
     if (e != cudaSuccess) {
-        (void)cudaGetLastError();
+        root->held -= (long long)cap;
+        pending.clear_later(h);
         h->last_err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
         throw Fail{PSSD_ERR_ALLOC};
     }
@@ -1605,12 +1632,15 @@ pssd_handle_s *acquire_helper(pssd_handle h)
         return x;
     }
     if ((int)root->helpers.size() >= MAX_HELPERS) return nullptr;
-    auto *x = new pssd_handle_s();
-    if (cudaStreamCreateWithFlags(&x->stream, cudaStreamNonBlocking) != cudaSuccess) {
-        (void)cudaGetLastError();
-        delete x;
+    const PendingError pending;
+    cudaStream_t stream;
+    if (cudaStreamCreateWithFlags(&stream, root->fault[PSSD_FAULT_STREAM] ? ~0u : cudaStreamNonBlocking) !=
+        cudaSuccess) {
+        pending.clear_later(h);
         return nullptr;
     }
+    auto *x = new pssd_handle_s();
+    x->stream = stream;
     x->root = root;
     x->chunk_bytes = size_t(1) << 28;
     root->helpers.push_back(x);
@@ -1630,8 +1660,7 @@ void free_idle_helpers(pssd_handle h)
     std::lock_guard<std::mutex> lk(root->helper_mu);
     for (auto *x : root->idle_helpers) {
         cudaStreamSynchronize(x->stream);
-        for (auto &c : x->chunks) if (c.owned) cudaFree(c.base);
-        x->chunks.clear();
+        free_chunks(x);
     }
 }
 
@@ -1644,7 +1673,9 @@ int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, in
 {
     int da = *maxdepth, db = *maxdepth;
     const Mark before = mark(h);
-    pssd_handle_s *x = std::min(a.m, b.m) > leaf ? acquire_helper(h) : nullptr;
+    const bool worth = std::min(a.m, b.m) > leaf;
+    if (worth && (root_of(h)->fault[PSSD_FAULT_LAUNCH] & 2)) refused_launch(h->stream);
+    pssd_handle_s *x = worth ? acquire_helper(h) : nullptr;
     std::thread second;
     cudaEvent_t done = nullptr;
     int st_b = PSSD_OK;
@@ -1660,7 +1691,7 @@ int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, in
             second = std::thread([&, dev, ready, done]() {
                 cudaSetDevice(dev);
                 Mark mk = mark(x);
-                if (x->root->fault[PSSD_FAULT_LAUNCH]) refused_launch(x->stream);
+                if (x->root->fault[PSSD_FAULT_LAUNCH] & 1) refused_launch(x->stream);
                 try {
                     cuda_check(x, cudaStreamWaitEvent(x->stream, ready, 0), "cudaStreamWaitEvent");
                     st_b = sym_eig_node(x, b.B, b.m, b.W, b.w, leaf, depth, &db, b.seed);
@@ -2106,7 +2137,7 @@ static void drop_helpers(pssd_handle h)
     for (auto *x : h->helpers) {
         cudaStreamSynchronize(x->stream);
         drop_side(x);
-        for (auto &c : x->chunks) if (c.owned) cudaFree(c.base);
+        free_chunks(x);
         for (auto &e : x->free_events) cudaEventDestroy(e);
         cudaStreamDestroy(x->stream);
         delete x;
@@ -2123,14 +2154,14 @@ int pssd_destroy(pssd_handle h)
         cudaStreamSynchronize(w->stream);
         drop_helpers(w);
         drop_side(w);
-        for (auto &c : w->chunks) if (c.owned) cudaFree(c.base);
+        free_chunks(w);
         for (auto &e : w->free_events) cudaEventDestroy(e);
         cudaStreamDestroy(w->stream);
         delete w;
     }
     drop_helpers(h);
     drop_side(h);
-    for (auto &c : h->chunks) if (c.owned) cudaFree(c.base);
+    free_chunks(h);
     for (auto &e : h->free_events) cudaEventDestroy(e);
     for (auto &e : h->events) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
     delete h;
@@ -2467,8 +2498,7 @@ int pssd_set_workspace(pssd_handle h, void *dptr, size_t bytes)
         return PSSD_ERR_CUDA;
     }
     drop_helpers(h);
-    for (auto &c : h->chunks) if (c.owned) cudaFree(c.base);
-    h->chunks.clear();
+    free_chunks(h);
     h->user_ws = false;
     h->depth = 0;
     h->peak = 0;

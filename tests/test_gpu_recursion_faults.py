@@ -37,3 +37,21 @@ def test_refused_launch_in_the_second_half_is_reported(P, call):
     D1, V1, _ = run()
     assert torch.equal(D1, D) and torch.equal(V1, V)
     h.close()
+
+
+@pytest.mark.parametrize("fault,value,launch", [("FAULT_MEMORY", 1 << 30, 1), ("FAULT_STREAM", 1, 2)])
+def test_refused_launch_survives_a_refused_helper(P, fault, value, launch):
+    """A second half without memory or stream runs in the first one's chain; a launch refused before is reported all
+    the same."""
+    H = _H(200)
+    h = P.Handle()
+    h.test_fault(getattr(P, fault), value)      # (1 GiB: the handle's own workspace, nothing for a helper)
+    D, V, _ = P.eig(H, handle=h)
+    h.test_fault(P.FAULT_LAUNCH, launch)
+    with pytest.raises(P.PssdError) as e:
+        P.eig(H, handle=h)
+    assert e.value.status == 6
+    h.test_fault(P.FAULT_LAUNCH, 0)
+    D1, V1, _ = P.eig(H, handle=h)
+    assert torch.equal(D1, D) and torch.equal(V1, V)
+    h.close()
