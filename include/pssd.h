@@ -167,9 +167,17 @@ const char *pssd_status_string(int status);
  * allocates, and a call that needs more returns PSSD_ERR_ALLOC (the handle
  * stays usable).  The worker handles of pssd_eig_batched keep library-managed
  * workspaces.
+ * The calls that diagonalise (pssd_eig, pssd_casida_eig, pssd_zeig, pssd_sign_vjp,
+ * pssd_gsplit) run the two halves of a division side by side, on up to three host
+ * threads with a stream and a workspace each beside the caller's.  Those
+ * workspaces come on top of the figures below and are kept with the handle; they
+ * are given back when an allocation of the handle fails, and with pssd_set_workspace
+ * and pssd_destroy, and a half that finds no memory beside the other runs after it,
+ * so a call needs no more than the figures below.  With a caller's buffer the halves
+ * run one after the other on the caller's thread.
  * ------------------------------------------------------------------------- */
-/* Upper bound on the workspace bytes of one pssd_sign / pssd_split / pssd_eig
- * call of order n with these options (r = 0 counts r = 8): (20 + 3 r) n^2
+/* Upper bound on the workspace bytes that one pssd_sign / pssd_split / pssd_eig
+ * call of order n needs with these options (r = 0 counts r = 8): (20 + 3 r) n^2
  * doubles + 256 MiB.  Returns -2 for n outside [1, PSSD_MAX_N]. */
 int pssd_workspace_bytes(pssd_handle h, int n, const pssd_opts *opts, size_t *bytes);
 /* Use [dptr, dptr + bytes) (device memory, at least 4096 bytes, owned by the
@@ -178,8 +186,8 @@ int pssd_workspace_bytes(pssd_handle h, int n, const pssd_opts *opts, size_t *by
  * workspace.  Synchronises the handle's stream and frees any workspace the
  * library had allocated; resets the peak. */
 int pssd_set_workspace(pssd_handle h, void *dptr, size_t bytes);
-/* Largest workspace (bytes) a call on this handle has needed since it was
- * created or since pssd_set_workspace: the exact size a caller-owned buffer
+/* Largest workspace (bytes) a call on this handle has needed, its halves taken one
+ * after the other, since it was created or since pssd_set_workspace: the exact size a caller-owned buffer
  * needs for the same calls. */
 int pssd_workspace_peak(pssd_handle h, size_t *bytes);
 
@@ -512,11 +520,13 @@ int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W,
  *                      looks for a helper, 3: both
  *   PSSD_FAULT_MEMORY  bytes that the workspaces of the handle and of its helpers may take
  *                      together: an allocation beyond is refused by the runtime
- *   PSSD_FAULT_STREAM  1: the runtime refuses the streams of new helpers */
+ *   PSSD_FAULT_STREAM  1: the runtime refuses the streams of new helpers
+ *   PSSD_FAULT_CHUNK   bytes of the smallest piece of workspace that is allocated at a time */
 #define PSSD_FAULT_LAUNCH 0
 #define PSSD_FAULT_MEMORY 1
 #define PSSD_FAULT_STREAM 2
-#define PSSD_FAULT_COUNT 3
+#define PSSD_FAULT_CHUNK 3
+#define PSSD_FAULT_COUNT 4
 int pssd_test_fault(pssd_handle h, int what, long long value);
 
 /* ---------------------------------------------------------------------------

@@ -149,6 +149,34 @@ struct PendingError {
     }
 };
 
+// a new chunk of at least `bytes`
+cudaError_t new_chunk(pssd_handle h, size_t bytes, Chunk &c)
+{
+    pssd_handle_s *root = root_of(h);
+    const size_t least = root->fault[PSSD_FAULT_CHUNK] ? (size_t)root->fault[PSSD_FAULT_CHUNK] : h->chunk_bytes;
+    c = {nullptr, std::max(bytes, least), bytes, true};
+    g_device_allocs.fetch_add(1, std::memory_order_relaxed);
+    const long long limit = root->fault[PSSD_FAULT_MEMORY], held = root->held += (long long)c.cap;
+    const cudaError_t e = cudaMalloc((void **)&c.base, limit && held > limit ? size_t(1) << 60 : c.cap);
+    if (e != cudaSuccess) root->held -= (long long)c.cap;
+    return e;
+}
+
+// gives the workspaces of helpers at rest back to the device; false if they hold none
+bool free_idle_helpers(pssd_handle h)
+{
+    pssd_handle_s *root = root_of(h);
+    std::lock_guard<std::mutex> lk(root->helper_mu);
+    bool any = false;
+    for (auto *x : root->idle_helpers) {
+        if (x->chunks.empty()) continue;
+        cudaStreamSynchronize(x->stream);
+        free_chunks(x);
+        any = true;
+    }
+    return any;
+}
+
 void *walloc(pssd_handle h, size_t bytes)
 {
     bytes = (bytes + 255) & ~size_t(255);
@@ -173,21 +201,21 @@ void *walloc(pssd_handle h, size_t bytes)
         size_t off = (i == m.chunk) ? c.off : 0;
         if (off + bytes <= c.cap) { c.off = off + bytes; return c.base + off; }
     }
-    size_t cap = std::max(bytes, h->chunk_bytes);
-    void *p = nullptr;
-    g_device_allocs.fetch_add(1, std::memory_order_relaxed);
     const PendingError pending;
-    pssd_handle_s *root = root_of(h);
-    const long long limit = root->fault[PSSD_FAULT_MEMORY], held = root->held += (long long)cap;
-    cudaError_t e = cudaMalloc(&p, limit && held > limit ? size_t(1) << 60 : cap);
+    Chunk c;
+    cudaError_t e = new_chunk(h, bytes, c);
+    // what helpers keep from earlier divisions goes before the call does
+    while (e == cudaErrorMemoryAllocation && free_idle_helpers(h)) {
+        pending.clear_later(h);
+        e = new_chunk(h, bytes, c);
+    }
     if (e != cudaSuccess) {
-        root->held -= (long long)cap;
         pending.clear_later(h);
         h->last_err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
         throw Fail{PSSD_ERR_ALLOC};
     }
-    h->chunks.push_back({(char *)p, cap, bytes, true});
-    return p;
+    h->chunks.push_back(c);
+    return c.base;
 }
 
 double *dalloc(pssd_handle h, size_t count) { return (double *)walloc(h, count * sizeof(double)); }
@@ -1651,17 +1679,6 @@ void give_back_helper(pssd_handle_s *x)
 {
     std::lock_guard<std::mutex> lk(x->root->helper_mu);
     x->root->idle_helpers.push_back(x);
-}
-
-// memory that helpers at rest hold
-void free_idle_helpers(pssd_handle h)
-{
-    pssd_handle_s *root = root_of(h);
-    std::lock_guard<std::mutex> lk(root->helper_mu);
-    for (auto *x : root->idle_helpers) {
-        cudaStreamSynchronize(x->stream);
-        free_chunks(x);
-    }
 }
 
 // The two halves of a division are independent, and below order 1000 or so neither fills the

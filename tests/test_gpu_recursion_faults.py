@@ -55,3 +55,54 @@ def test_refused_launch_survives_a_refused_helper(P, fault, value, launch):
     D1, V1, _ = P.eig(H, handle=h)
     assert torch.equal(D1, D) and torch.equal(V1, V)
     h.close()
+
+
+MIB = 1 << 20
+
+
+def _program(P, cap, side_by_side, kind, H, h=None):
+    """The outputs of a program whose last call may use `cap` bytes of workspace (0: no limit); None if they are too
+    few.  Pieces of 1 MiB, so that what is held follows what is needed."""
+    k = H.shape[0] // 2
+    own = h is None
+    if own:
+        h = P.Handle()
+        h.test_fault(P.FAULT_CHUNK, MIB)
+        h.test_fault(P.FAULT_STREAM, 0 if side_by_side else 1)
+    if kind == "eig then split":
+        P.eig(H, handle=h)
+    h.test_fault(P.FAULT_MEMORY, cap)
+    try:
+        if kind == "eig":
+            out = P.eig(H, handle=h)[:2]
+        elif kind == "casida_eig":
+            out = P.casida_eig(H[:k, :k].contiguous(), H[:k, k:].contiguous(), handle=h)[:2]
+        else:
+            out = P.split(H, r=8, handle=h, precision=P.PSSD_FP64_EMULATED)[:3]
+    except P.PssdError as e:
+        assert e.status == 7
+        out = None
+    h.test_fault(P.FAULT_MEMORY, 0)
+    if own:
+        h.close()
+    return out
+
+
+@pytest.mark.parametrize("kind", ["eig", "casida_eig", "eig then split"])
+def test_what_fits_in_sequence_fits_side_by_side(P, kind):
+    """The least memory with which a program runs without helpers is enough with them, and so is anything between
+    that and what it takes undisturbed; the results are the same to the bit."""
+    H = _H(260)
+    ref = _program(P, 0, False, kind, H)
+    lo, hi = 0, 4096                                 # MiB: too little, enough
+    assert _program(P, hi * MIB, False, kind, H) is not None
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        if _program(P, mid * MIB, False, kind, H) is None:
+            lo = mid
+        else:
+            hi = mid
+    for cap in [hi * MIB + d * MIB for d in (0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 64, 128)] + [0]:
+        out = _program(P, cap, True, kind, H)
+        assert out is not None, (hi, cap // MIB)
+        assert all(torch.equal(x, y) for x, y in zip(out, ref)), cap // MIB
