@@ -170,11 +170,11 @@ const char *pssd_status_string(int status);
  * The calls that diagonalise (pssd_eig, pssd_casida_eig, pssd_zeig, pssd_sign_vjp,
  * pssd_gsplit) run the two halves of a division side by side, on up to three host
  * threads with a stream and a workspace each beside the caller's.  Those
- * workspaces come on top of the figures below and are kept with the handle; they
- * are given back when an allocation of the handle fails, and with pssd_set_workspace
- * and pssd_destroy, and a half that finds no memory beside the other runs after it,
- * so a call needs no more than the figures below.  With a caller's buffer the halves
- * run one after the other on the caller's thread.
+ * workspaces come on top of the figures below; 1 GiB of each is kept with the
+ * handle after a call and given back when an allocation of the handle fails and with
+ * pssd_set_workspace and pssd_destroy.  A half that finds no memory beside the other
+ * runs after it, so a call needs no more than the figures below.  With a caller's
+ * buffer the halves run one after the other on the caller's thread.
  * ------------------------------------------------------------------------- */
 /* Upper bound on the workspace bytes that one pssd_sign / pssd_split / pssd_eig
  * call of order n needs with these options (r = 0 counts r = 8): (20 + 3 r) n^2

@@ -127,15 +127,17 @@ void release(pssd_handle h, Mark m)
     h->depth = m.depth;
 }
 
-// the handle's own chunks
-void free_chunks(pssd_handle h)
+// the handle's own chunks, but for the first ones up to `keep` bytes
+void free_chunks(pssd_handle h, size_t keep = 0)
 {
-    for (auto &c : h->chunks)
-        if (c.owned) {
-            cudaFree(c.base);
-            root_of(h)->held -= (long long)c.cap;
+    size_t n = 0, sum = 0;
+    while (n < h->chunks.size() && sum + h->chunks[n].cap <= keep) sum += h->chunks[n++].cap;
+    for (size_t i = n; i < h->chunks.size(); ++i)
+        if (h->chunks[i].owned) {
+            cudaFree(h->chunks[i].base);
+            root_of(h)->held -= (long long)h->chunks[i].cap;
         }
-    h->chunks.clear();
+    h->chunks.resize(n);
 }
 
 // A launch refused earlier in the call, which the check at its end reports, before a call whose
@@ -162,16 +164,19 @@ cudaError_t new_chunk(pssd_handle h, size_t bytes, Chunk &c)
     return e;
 }
 
-// gives the workspaces of helpers at rest back to the device; false if they hold none
-bool free_idle_helpers(pssd_handle h)
+// Gives the workspaces of helpers at rest back to the device, but for `keep` bytes of each; false
+// if there is nothing to give back.
+bool free_idle_helpers(pssd_handle h, size_t keep = 0)
 {
     pssd_handle_s *root = root_of(h);
     std::lock_guard<std::mutex> lk(root->helper_mu);
     bool any = false;
     for (auto *x : root->idle_helpers) {
-        if (x->chunks.empty()) continue;
+        size_t sum = 0;
+        for (const Chunk &c : x->chunks) sum += c.cap;
+        if (sum <= keep) continue;
         cudaStreamSynchronize(x->stream);
-        free_chunks(x);
+        free_chunks(x, keep);
         any = true;
     }
     return any;
@@ -1644,6 +1649,10 @@ int sym_eig(pssd_handle h, const double *B, int m, double *W, double *w, int lea
 
 constexpr int MAX_HELPERS = 3;
 
+// What a helper keeps of its workspace from call to call.  An eig of order 4096 needs 0.75 GB in
+// each, one of 16384 15 GB, which the caller's program may want between two calls.
+constexpr size_t HELPER_KEEP = size_t(1) << 30;
+
 // a launch that the runtime refuses (no such block size), for pssd_test_fault
 __global__ void refused_kernel() {}
 void refused_launch(cudaStream_t s) { refused_kernel<<<1, 4096, 0, s>>>(); }
@@ -2107,7 +2116,10 @@ int guarded(pssd_handle h, pssd_info *info, F body)
     } catch (Fail &f) {
         st = f.code;
     }
-    if (!outer_err) h->derr = nullptr;
+    if (!outer_err) {
+        h->derr = nullptr;
+        free_idle_helpers(h, HELPER_KEEP);
+    }
     if (h->side) cudaStreamSynchronize(h->side);   // leaves still running on an error path
     h->leaf_pending.clear();
     h->sync_used = 0;

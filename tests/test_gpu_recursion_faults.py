@@ -106,3 +106,28 @@ def test_what_fits_in_sequence_fits_side_by_side(P, kind):
         out = _program(P, cap, True, kind, H)
         assert out is not None, (hi, cap // MIB)
         assert all(torch.equal(x, y) for x, y in zip(out, ref)), cap // MIB
+
+
+def test_helpers_keep_little_between_calls(P):
+    """After a large call the helpers hold 1 GiB each at most beside what the handle keeps without them."""
+    n = 8192
+    g = torch.Generator(device="cuda"); g.manual_seed(2)
+    B = torch.randn(n, n, device="cuda", dtype=torch.float64, generator=g)
+    M = B @ B.T / n + torch.eye(n, device="cuda", dtype=torch.float64)
+    s = torch.ones(n, device="cuda", dtype=torch.float64)
+    s[1::2] = -1.0
+    H, sigma = s[:, None] * (0.5 * (M + M.T)), s.cpu().numpy()
+    del B, M
+    small = _H(200)
+    kept = []
+    for refused in (1, 0):
+        h = P.Handle()
+        h.test_fault(P.FAULT_STREAM, refused)
+        P.eig(small, handle=h)                       # (loads the kernels)
+        P.eig(H, sigma=sigma, handle=h, precision=P.PSSD_FP64_EMULATED)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        before = torch.cuda.mem_get_info()[0]
+        h.close()
+        kept.append(torch.cuda.mem_get_info()[0] - before)
+    assert kept[1] - kept[0] <= 3 * 1024 * MIB + 64 * MIB, kept
