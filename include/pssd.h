@@ -52,7 +52,7 @@ extern "C" {
 #define PSSD_ERR_NO_CONVERGENCE 2      /* Alg. 8 stopping test still failing after max_restarts restarts */
 #define PSSD_ERR_BASIS 3               /* split: basis rank or orthogonalisation breakdown */
 #define PSSD_ERR_NONFINITE 4           /* NaN/Inf in the input or an iterate */
-#define PSSD_ERR_TIMEOUT 5             /* a bounded device wait gave up (tensor-core pipeline) */
+#define PSSD_ERR_TIMEOUT 5             /* a bounded wait inside a kernel gave up */
 #define PSSD_ERR_CUDA 6                /* a CUDA call failed; see pssd_last_cuda_error */
 #define PSSD_ERR_ALLOC 7               /* workspace allocation failed, or the caller's workspace is too small */
 #define PSSD_ERR_NOT_PSEUDOSYMMETRIC 8 /* ||Sigma H - (Sigma H)^T||_F > 1e-12 ||Sigma H||_F */
@@ -521,12 +521,16 @@ int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W,
  *   PSSD_FAULT_MEMORY  bytes that the workspaces of the handle and of its helpers may take
  *                      together: an allocation beyond is refused by the runtime
  *   PSSD_FAULT_STREAM  1: the runtime refuses the streams of new helpers
- *   PSSD_FAULT_CHUNK   bytes of the smallest piece of workspace that is allocated at a time */
+ *   PSSD_FAULT_CHUNK   bytes of the smallest piece of workspace that is allocated at a time
+ *   PSSD_FAULT_LEAF64_WAIT, PSSD_FAULT_LEAF32_WAIT  1: the waits inside the FP64 and FP32
+ *                      Cholesky leaves run out at their first poll */
 #define PSSD_FAULT_LAUNCH 0
 #define PSSD_FAULT_MEMORY 1
 #define PSSD_FAULT_STREAM 2
 #define PSSD_FAULT_CHUNK 3
-#define PSSD_FAULT_COUNT 4
+#define PSSD_FAULT_LEAF64_WAIT 4
+#define PSSD_FAULT_LEAF32_WAIT 5
+#define PSSD_FAULT_COUNT 6
 int pssd_test_fault(pssd_handle h, int what, long long value);
 
 /* ---------------------------------------------------------------------------

@@ -51,4 +51,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
     return done != 0;
 }
 
+// The same for a barrier's first phase, with a bound known at compile time: 1, or 0 on timeout.
+template <unsigned int LIMIT> __device__ __forceinline__ uint32_t mbar_wait_first(uint32_t bar)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], 0;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar)
+        : "memory");
+    for (unsigned int it = 1; !done && it < LIMIT; ++it)
+        asm volatile(
+            "{\n.reg .pred p;\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n"
+            "selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(bar)
+            : "memory");
+    return done;
+}
+
 }  // namespace pssd

@@ -71,7 +71,7 @@ struct pssd_handle_s {
     pssd_handle_s *root = nullptr;
     bool sequential = false;                // never use helpers (many batch workers run already)
     size_t chunk_bytes = size_t(1) << 30;   // smallest workspace chunk
-    int *derr = nullptr;    // device error flag of the current call (bounded waits in the tensor-core kernel)
+    int *derr = nullptr;    // device error flag of the current call (bounded waits inside the kernels)
     int use_tc = 1;         // FP32 contractions on tcgen05 tensor cores (0: FP32 SIMT kernel)
     int force_engine = 0;   // test hooks: no size-based engine selection
     bool pinned = false;    // products upstream of the mixed mode's FP32 stage (see gemm())
@@ -477,7 +477,8 @@ void chol_rec(pssd_handle h, T *A, int off, int s, long long lda, long long sA, 
 {
     if (s <= CholLeaf<T>::max_s) {
         Timed t(h, K_CHOL_LEAF, batch * (double)s * s * s);
-        if (chol_leaf<T>(A, lda, sA, Rinv, lda, sR, off, s, batch, dinfo, h->stream)) {
+        const bool one_poll = root_of(h)->fault[sizeof(T) == 8 ? PSSD_FAULT_LEAF64_WAIT : PSSD_FAULT_LEAF32_WAIT] != 0;
+        if (chol_leaf<T>(A, lda, sA, Rinv, lda, sR, off, s, batch, dinfo, h->derr, one_poll, h->stream)) {
             h->last_err = "Cholesky leaf launch configuration failed";
             throw Fail{PSSD_ERR_CUDA};
         }
@@ -2109,7 +2110,7 @@ int guarded(pssd_handle h, pssd_info *info, F body)
             int herr = 0;
             cudaMemcpyAsync(&herr, h->derr, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
             cudaStreamSynchronize(h->stream);
-            // a tensor-core kernel that gave up leaves garbage behind it, so the later
+            // a kernel that gave up a wait leaves garbage behind it, so the later
             // steps may fail too; the timeout is the cause that is reported
             if (herr && st != PSSD_ERR_CUDA) st = PSSD_ERR_TIMEOUT;
         }

@@ -94,14 +94,15 @@ double oz_gemm_time_us(const GemmArgs &g);   // estimated time of both
 // of each batch matrix, in one launch: L (lower) in place in A with zeros
 // above the diagonal inside the block, L^{-1} (lower) in the same block of
 // Rinv.  info[z] = (first failing global pivot + 1) if a pivot is not
-// positive or finite (the factorisation then continues with pivot 1).
+// positive or finite (the factorisation then continues with pivot 1).  A wait inside the
+// kernel that runs out (one_poll: at its first poll) sets *err (may be null) and info[z].
 // s <= CholLeaf<T>::max_s; returns nonzero on a launch-configuration error.
 template <class T> struct CholLeaf;
 template <> struct CholLeaf<float> { static constexpr int max_s = 128; };
 template <> struct CholLeaf<double> { static constexpr int max_s = 64; };
 template <class T>
 int chol_leaf(T *A, long long lda, long long sA, T *Rinv, long long ldr, long long sR, int off, int s, int batch,
-              int *info, cudaStream_t st);
+              int *info, int *err, bool one_poll, cudaStream_t st);
 
 // Elementwise / HBM passes
 void sym_prepare(const double *H, long long ldh, const double *sig, int n, double *M, long long ldm,
