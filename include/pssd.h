@@ -523,14 +523,16 @@ int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W,
  *   PSSD_FAULT_STREAM  1: the runtime refuses the streams of new helpers
  *   PSSD_FAULT_CHUNK   bytes of the smallest piece of workspace that is allocated at a time
  *   PSSD_FAULT_LEAF64_WAIT, PSSD_FAULT_LEAF32_WAIT  1: the waits inside the FP64 and FP32
- *                      Cholesky leaves run out at their first poll */
+ *                      Cholesky leaves run out at their first poll
+ *   PSSD_FAULT_KRYLOV_WAIT  bound on the waits inside the one-launch Krylov loops, in polls */
 #define PSSD_FAULT_LAUNCH 0
 #define PSSD_FAULT_MEMORY 1
 #define PSSD_FAULT_STREAM 2
 #define PSSD_FAULT_CHUNK 3
 #define PSSD_FAULT_LEAF64_WAIT 4
 #define PSSD_FAULT_LEAF32_WAIT 5
-#define PSSD_FAULT_COUNT 6
+#define PSSD_FAULT_KRYLOV_WAIT 6
+#define PSSD_FAULT_COUNT 7
 int pssd_test_fault(pssd_handle h, int what, long long value);
 
 /* ---------------------------------------------------------------------------

@@ -1899,8 +1899,10 @@ void dot_vec(const double *x, const double *y, int n, double *out, cudaStream_t 
 // memory to every CTA (two buffers in turn) behind one grid barrier; the dot
 // products, the three-term update and the normalisation are then done by every
 // CTA for itself, in the same order, so all hold the same bits.  The launch is
-// cooperative -- all CTAs are resident before any waits -- and a wait that runs
-// out of polls makes the loop return NaN.
+// cooperative -- all CTAs are resident before any waits.  A CTA whose wait runs
+// out of polls leaves without another arrival, so that nobody passes a later
+// barrier: CTA 0, which writes the results, either passed every barrier or gives up
+// as well, writes NaN and sets the error flag.
 // Sums: 32 consecutive entries by a shuffle tree, the trees' results in order,
 // over KRY_SEGMENTS equal segments of the vector first, then those in order.
 // Measured, 24 Lanczos steps: m = 128 190 us, m = 1000 400 us; on one cluster of 8
@@ -1909,10 +1911,10 @@ void dot_vec(const double *x, const double *y, int n, double *out, cudaStream_t 
 constexpr int KRY_ROWS = 8, KRY_THREADS = 32 * KRY_ROWS, KRY_SEGMENTS = 8;
 constexpr int KRY_T = KRY_MAX_M / 32;                  // entries of a row per lane
 constexpr int KRY_GROUPS = KRY_SEGMENTS * (KRY_MAX_M / KRY_SEGMENTS / 32);   // sums of 32 entries, at most
-constexpr unsigned int KRY_WAIT_LIMIT = 1u << 22;
+constexpr unsigned int KRY_WAIT_LIMIT = 1u << 22;      // default bound of a wait, in polls
 
 // every CTA of the grid has arrived (count: 0 at launch; target: arrivals so far times CTAs)
-__device__ __forceinline__ bool kry_grid_sync(unsigned int *count, unsigned int target, int *sm_ok)
+__device__ __forceinline__ bool kry_grid_sync(unsigned int *count, unsigned int target, unsigned int limit, int *sm_ok)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1920,7 +1922,7 @@ __device__ __forceinline__ bool kry_grid_sync(unsigned int *count, unsigned int 
         __threadfence();
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
         int ok = 0;
-        for (unsigned int it = 0; it < KRY_WAIT_LIMIT; ++it) {
+        for (unsigned int it = 0; it < limit; ++it) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
             if (v >= target) { ok = 1; break; }
         }
@@ -1995,7 +1997,7 @@ __device__ __forceinline__ double kry_row_dot(const double *row, int len, const 
 template <int OP>
 __global__ void __launch_bounds__(KRY_THREADS, 1)
 krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps, int power, uint64_t seed, double *out,
-                   double *ex, unsigned int *count)
+                   double *ex, unsigned int *count, int *err, unsigned int limit)
 {
     __shared__ double cur[KRY_MAX_M], prv[KRY_MAX_M], w[KRY_MAX_M];
     __shared__ double red[KRY_GROUPS + 8], bc[2];
@@ -2005,16 +2007,24 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
     const int seg = (m + KRY_SEGMENTS - 1) / KRY_SEGMENTS;
     unsigned int arrived = 0;
     int turn = 0;
-    bool ok = true;
-    // entry r of a vector (lane 0's v) -> dst, whole in every CTA
-    auto exchange = [&](double v, double *dst) {
+    // entry r of a vector (lane 0's v) -> dst, whole in every CTA; false if a wait ran out
+    auto exchange = [&](double v, double *dst) -> bool {
         double *buf = ex + turn * m;
         turn ^= 1;
         if (r < m && lane == 0) __stcg(buf + r, v);
         arrived += gridDim.x;
-        if (ok) ok = kry_grid_sync(count, arrived, &sm_ok);
+        if (!kry_grid_sync(count, arrived, limit, &sm_ok)) return false;
         for (int i = tid; i < m; i += KRY_THREADS) dst[i] = __ldcg(buf + i);
         __syncthreads();
+        return true;
+    };
+    auto give_up = [&]() {
+        if (blockIdx.x != 0 || tid != 0) return;
+        for (int j = 0; j < (power > 0 ? 1 : steps); ++j) {
+            out[j] = NAN;
+            if (power == 0) out[steps + 1 + j] = NAN;
+        }
+        if (err) atomicExch(err, 6);
     };
     // this warp's row of A (of L), and column of L
     const int rlen = r < m ? (OP == KRY_SYM ? m : r + 1) : 0;
@@ -2025,28 +2035,25 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
         row[t] = i < rlen ? __ldg(A + (long long)r * lda + i) : 0.0;
         if (OP == KRY_TRI_PAIR) col[t] = (r < m && i >= r && i < m) ? __ldg(A + (long long)i * lda + r) : 0.0;
     }
-    exchange(r < m && lane == 0 ? gauss_at(seed, (uint64_t)r) : 0.0, cur);
+    if (!exchange(r < m && lane == 0 ? gauss_at(seed, (uint64_t)r) : 0.0, cur)) return give_up();
     kry_sum(m, KRY_MAX_M, [&](int i) { return cur[i] * cur[i]; }, red, bc, true);
     const double inv0 = bc[1];
     for (int i = tid; i < m; i += KRY_THREADS) { cur[i] *= inv0; prv[i] = 0.0; }
     __syncthreads();
-    auto apply = [&]() {                               // op(A) cur -> w
-        if (OP == KRY_SYM) {
-            exchange(kry_row_dot(row, rlen, cur, lane), w);
-        } else {
-            exchange(kry_row_dot(row, rlen, cur, lane), w);                    // u = L x
-            exchange(kry_row_dot(col, r < m ? m : 0, w, lane), w);             // L^T u (zeros above the diagonal)
-        }
+    auto apply = [&]() -> bool {                       // op(A) cur -> w
+        if (!exchange(kry_row_dot(row, rlen, cur, lane), w)) return false;
+        // w = u = L x: L^T u (zeros above the diagonal)
+        return OP == KRY_SYM || exchange(kry_row_dot(col, r < m ? m : 0, w, lane), w);
     };
     if (power == 0) {
         double beta_prev = 0.0;
         for (int j = 0; j < steps; ++j) {
-            apply();
+            if (!apply()) return give_up();
             const double alpha = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, bc);
             for (int i = tid; i < m; i += KRY_THREADS) w[i] = w[i] - alpha * cur[i] - beta_prev * prv[i];
             __syncthreads();
             const double beta = kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, bc, true);
-            if (blockIdx.x == 0 && tid == 0) { out[j] = ok ? alpha : NAN; out[steps + 1 + j] = ok ? beta : NAN; }
+            if (blockIdx.x == 0 && tid == 0) { out[j] = alpha; out[steps + 1 + j] = beta; }
             const double scale = bc[1];
             for (int i = tid; i < m; i += KRY_THREADS) { prv[i] = cur[i]; cur[i] = w[i] * scale; }
             __syncthreads();
@@ -2054,27 +2061,28 @@ krylov_grid_kernel(const double *__restrict__ A, long long lda, int m, int steps
         }
     } else {
         for (int it = 0; it < power; ++it) {
-            apply();
+            if (!apply()) return give_up();
             kry_sum(m, seg, [&](int i) { return w[i] * w[i]; }, red, bc, true);
             const double scale = bc[1];
             for (int i = tid; i < m; i += KRY_THREADS) cur[i] = w[i] * scale;
             __syncthreads();
         }
-        apply();
+        if (!apply()) return give_up();
         const double rq = kry_sum(m, seg, [&](int i) { return cur[i] * w[i]; }, red, bc);
-        if (blockIdx.x == 0 && tid == 0) out[0] = ok ? rq : NAN;
+        if (blockIdx.x == 0 && tid == 0) out[0] = rq;
     }
 }
 
 size_t krylov_scratch_doubles(int m) { return 2 * (size_t)m + 8; }
 
 bool krylov_fused(const double *A, long long lda, int op, int m, int steps, int power, uint64_t seed, double *out,
-                  double *scratch, cudaStream_t s)
+                  double *scratch, int *err, unsigned int wait_limit, cudaStream_t s)
 {
     if (m < 1 || m > KRY_MAX_M || steps < 0 || power < 0) return false;
     unsigned int *count = (unsigned int *)(scratch + 2 * (size_t)m);
     if (cudaMemsetAsync(count, 0, sizeof(unsigned int), s) != cudaSuccess) return false;
-    void *args[] = {&A, &lda, &m, &steps, &power, &seed, &out, &scratch, &count};
+    unsigned int limit = wait_limit ? wait_limit : KRY_WAIT_LIMIT;
+    void *args[] = {&A, &lda, &m, &steps, &power, &seed, &out, &scratch, &count, &err, &limit};
     const void *kernel = op == KRY_SYM ? (const void *)krylov_grid_kernel<KRY_SYM>
                                        : (const void *)krylov_grid_kernel<KRY_TRI_PAIR>;
     if (cudaLaunchCooperativeKernel(kernel, dim3((m + KRY_ROWS - 1) / KRY_ROWS), dim3(KRY_THREADS), args, 0, s) !=

@@ -1025,7 +1025,8 @@ struct KryFused {
     {
         Mark mk = mark(h);
         double *scratch = dalloc(h, krylov_scratch_doubles(m));
-        if (!krylov_fused(A, lda, op, m, steps, power, seed, out, scratch, h->stream)) {
+        if (!krylov_fused(A, lda, op, m, steps, power, seed, out, scratch, h->derr,
+                          (unsigned int)root_of(h)->fault[PSSD_FAULT_KRYLOV_WAIT], h->stream)) {
             h->last_err = std::string("Krylov launch: ") + cudaGetErrorString(cudaGetLastError());
             throw Fail{PSSD_ERR_CUDA};
         }

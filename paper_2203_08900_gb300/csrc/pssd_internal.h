@@ -176,13 +176,14 @@ void lanczos_update(double *w, const double *v, const double *vprev, const doubl
 //   power == 0: `steps` Lanczos steps; out[j] = alpha_j (j < steps) and
 //               out[steps + 1 + j] = beta_j, the layout of the step-by-step loop.
 //   power  > 0: `power` normalised power steps, then out[0] = v^T A v.
-// scratch: krylov_scratch_doubles(m) doubles.  Returns false (nothing launched) if m is outside
+// scratch: krylov_scratch_doubles(m) doubles.  A wait inside the kernel of more than wait_limit
+// polls (0: the default) sets *err (may be null) and the results to NaN.  Returns false (nothing launched) if m is outside
 // [1, KRY_MAX_M] or the launch failed.
 constexpr int KRY_MAX_M = 1024;
 enum KryOp { KRY_SYM = 0, KRY_TRI_PAIR = 1 };
 size_t krylov_scratch_doubles(int m);
 bool krylov_fused(const double *A, long long lda, int op, int m, int steps, int power, uint64_t seed, double *out,
-                  double *scratch, cudaStream_t s);
+                  double *scratch, int *err, unsigned int wait_limit, cudaStream_t s);
 void scale_columns(double *X, long long ldx, int m, int n, const double *d, int use_sqrt_abs,
                    cudaStream_t s);
 void sign_fix_columns(double *X, long long ldx, int m, int n, cudaStream_t s);
