@@ -494,7 +494,7 @@ int pssd_gsplit(pssd_handle h, int n, const signed char *sigma, const double *H,
  * = beta_j (device, 2 steps + 2 doubles).  power > 0: that many normalised power
  * steps from the Gaussian vector of seed 0x5eed, then out[0] = v^T op(A) v.
  * fused = 0: one launch per vector operation; fused = 1: the whole loop in one
- * cooperative launch (m <= 1024).  v0 (device, m, or NULL) receives the
+ * cooperative launch (m <= 1024; step by step if that launch is refused).  v0 (device, m, or NULL) receives the
  * starting vector before normalisation.  Returns 0 or a negative argument index
  * (-6: power outside [0, 1000], or power = 0 with steps outside [1, m]). */
 #define PSSD_KRYLOV_SYM 0
@@ -524,7 +524,8 @@ int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W,
  *   PSSD_FAULT_CHUNK   bytes of the smallest piece of workspace that is allocated at a time
  *   PSSD_FAULT_LEAF64_WAIT, PSSD_FAULT_LEAF32_WAIT  1: the waits inside the FP64 and FP32
  *                      Cholesky leaves run out at their first poll
- *   PSSD_FAULT_KRYLOV_WAIT  bound on the waits inside the one-launch Krylov loops, in polls */
+ *   PSSD_FAULT_KRYLOV_WAIT  bound on the waits inside the one-launch Krylov loops, in polls
+ *   PSSD_FAULT_KRYLOV_LAUNCH  1: the launch of these loops is refused by the runtime */
 #define PSSD_FAULT_LAUNCH 0
 #define PSSD_FAULT_MEMORY 1
 #define PSSD_FAULT_STREAM 2
@@ -532,7 +533,8 @@ int pssd_test_sym_eig(pssd_handle h, int m, const double *B, int ldb, double *W,
 #define PSSD_FAULT_LEAF64_WAIT 4
 #define PSSD_FAULT_LEAF32_WAIT 5
 #define PSSD_FAULT_KRYLOV_WAIT 6
-#define PSSD_FAULT_COUNT 7
+#define PSSD_FAULT_KRYLOV_LAUNCH 7
+#define PSSD_FAULT_COUNT 8
 int pssd_test_fault(pssd_handle h, int what, long long value);
 
 /* ---------------------------------------------------------------------------

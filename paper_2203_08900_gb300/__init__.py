@@ -31,7 +31,7 @@ FLAG_NO_REFINE = 8
 FLAG_RECOMPUTE = 16
 METHOD_ZOLO, METHOD_DWH, METHOD_NEWTON = 0, 1, 2
 (FAULT_LAUNCH, FAULT_MEMORY, FAULT_STREAM, FAULT_CHUNK, FAULT_LEAF64_WAIT, FAULT_LEAF32_WAIT,
- FAULT_KRYLOV_WAIT) = range(7)
+ FAULT_KRYLOV_WAIT, FAULT_KRYLOV_LAUNCH) = range(8)
 
 
 class Opts(ctypes.Structure):

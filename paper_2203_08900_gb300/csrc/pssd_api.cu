@@ -140,6 +140,10 @@ void free_chunks(pssd_handle h, size_t keep = 0)
     h->chunks.resize(n);
 }
 
+// a launch that the runtime refuses (no such block size), for pssd_test_fault
+__global__ void refused_kernel() {}
+void refused_launch(cudaStream_t s) { refused_kernel<<<1, 4096, 0, s>>>(); }
+
 // A launch refused earlier in the call, which the check at its end reports, before a call whose
 // failure is dealt with here: the runtime keeps one error per thread, the latest.
 struct PendingError {
@@ -1021,43 +1025,49 @@ struct KryFused {
     long long lda = 0;
     int op = KRY_SYM;
     bool usable(int m) const { return A && m >= 1 && m <= KRY_MAX_M; }
-    void run(pssd_handle h, int m, int steps, int power, uint64_t seed, double *out) const
+    // false if the launch was refused: it needs all of its CTAs on the GPU at once, which a
+    // partition of the GPU may not give it
+    bool run(pssd_handle h, int m, int steps, int power, uint64_t seed, double *out) const
     {
+        const long long *fault = root_of(h)->fault;
+        const PendingError pending;
         Mark mk = mark(h);
         double *scratch = dalloc(h, krylov_scratch_doubles(m));
-        if (!krylov_fused(A, lda, op, m, steps, power, seed, out, scratch, h->derr,
-                          (unsigned int)root_of(h)->fault[PSSD_FAULT_KRYLOV_WAIT], h->stream)) {
-            h->last_err = std::string("Krylov launch: ") + cudaGetErrorString(cudaGetLastError());
-            throw Fail{PSSD_ERR_CUDA};
+        bool ok;
+        {
+            const double products = power > 0 ? power + 1 : steps;
+            Timed t(h, K_GEMV, products * 2.0 * m * (double)m, products * 8.0 * m * (double)m);
+            if (fault[PSSD_FAULT_KRYLOV_LAUNCH]) refused_launch(h->stream);
+            ok = !fault[PSSD_FAULT_KRYLOV_LAUNCH] &&
+                 krylov_fused(A, lda, op, m, steps, power, seed, out, scratch, h->derr,
+                              (unsigned int)fault[PSSD_FAULT_KRYLOV_WAIT], h->stream);
         }
         release(h, mk);
+        if (!ok) pending.clear_later(h);
+        return ok;
     }
 };
 
 // power iteration estimate of lambda_max of an SPD operator given by `apply` (or by `kf`:
-// the same iteration in one launch, the same starting vector)
+// the same iteration in one launch, unless that is refused, the same starting vector)
 template <class F>
 void power_device(pssd_handle h, int n, F apply, double *v, double *w, double *dscal, int iters,
                   const KryFused *kf = nullptr)
 {
-    if (kf && kf->usable(n) && iters > 0) {
-        Timed t(h, K_GEMV, (iters + 1) * 2.0 * n * (double)n, (iters + 1) * 8.0 * n * (double)n);
-        kf->run(h, n, 0, iters, 0x5eedull, dscal);
-    } else {
-        {
-            Timed t(h, K_HBM, 0, 24.0 * n);
-            fill_gaussian(v, n, 1, n, 0x5eedull, h->stream);
-            normalize_vec(v, v, n, nullptr, h->stream);
-        }
-        for (int it = 0; it < iters; ++it) {
-            apply(v, w);
-            Timed t(h, K_GEMV, 0, 16.0 * n);
-            normalize_vec(w, v, n, nullptr, h->stream);
-        }
+    if (kf && kf->usable(n) && iters > 0 && kf->run(h, n, 0, iters, 0x5eedull, dscal)) return;
+    {
+        Timed t(h, K_HBM, 0, 24.0 * n);
+        fill_gaussian(v, n, 1, n, 0x5eedull, h->stream);
+        normalize_vec(v, v, n, nullptr, h->stream);
+    }
+    for (int it = 0; it < iters; ++it) {
         apply(v, w);
         Timed t(h, K_GEMV, 0, 16.0 * n);
-        dot_vec(v, w, n, dscal, h->stream);
+        normalize_vec(w, v, n, nullptr, h->stream);
     }
+    apply(v, w);
+    Timed t(h, K_GEMV, 0, 16.0 * n);
+    dot_vec(v, w, n, dscal, h->stream);
 }
 
 template <class F>
@@ -1338,14 +1348,11 @@ void small_sym_eig(std::vector<double> A, int n, std::vector<double> &w, std::ve
 // recurrence produced a non-finite value.
 // `steps` Lanczos steps from the seeded Gaussian vector: ab[j] = alpha_j, ab[steps + 1 + j] =
 // beta_j (device), step by step through `apply`, or in one launch through `kf` when m fits it
+// and the launch is not refused
 template <class F>
 void lanczos_device(pssd_handle h, int m, F apply, uint64_t seed, int steps, double *ab, const KryFused *kf)
 {
-    if (kf && kf->usable(m)) {
-        Timed t(h, K_GEMV, steps * 2.0 * m * (double)m, steps * 8.0 * m * (double)m);
-        kf->run(h, m, steps, 0, seed, ab);
-        return;
-    }
+    if (kf && kf->usable(m) && kf->run(h, m, steps, 0, seed, ab)) return;
     Mark mk = mark(h);
     double *V = dalloc(h, 3 * (size_t)m);
     double *vp = V, *vc = V + m, *w = V + 2 * m;
@@ -1654,10 +1661,6 @@ constexpr int MAX_HELPERS = 3;
 // What a helper keeps of its workspace from call to call.  An eig of order 4096 needs 0.75 GB in
 // each, one of 16384 15 GB, which the caller's program may want between two calls.
 constexpr size_t HELPER_KEEP = size_t(1) << 30;
-
-// a launch that the runtime refuses (no such block size), for pssd_test_fault
-__global__ void refused_kernel() {}
-void refused_launch(cudaStream_t s) { refused_kernel<<<1, 4096, 0, s>>>(); }
 
 // an idle helper of h's calling handle, or null: none left, or workspace that may not grow
 pssd_handle_s *acquire_helper(pssd_handle h)
