@@ -601,6 +601,9 @@ int pssd_launch_count_phases(long long *counts, int n);
 /* Number of device allocations (cudaMalloc calls) the library has made in this
  * process (all handles, workspace growth included). */
 long long pssd_device_alloc_count(void);
+/* Number of CUDA events the library has made for profiling in this process (they are
+ * pooled, so it stops growing when calls of one kind repeat). */
+long long pssd_timing_event_count(void);
 
 #ifdef __cplusplus
 }

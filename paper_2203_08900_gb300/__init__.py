@@ -74,7 +74,8 @@ EXPORTS = ["pssd_opts_init", "pssd_create", "pssd_destroy", "pssd_set_stream", "
            "pssd_test_gemm_f64", "pssd_workspace_bytes", "pssd_set_workspace", "pssd_workspace_peak",
            "pssd_device_alloc_count", "pssd_casida_sign", "pssd_casida_split", "pssd_casida_eig",
            "pssd_test_sym_eig", "pssd_sign_vjp_rev", "pssd_zsign", "pssd_zeig", "pssd_launch_count_phases",
-           "pssd_test_krylov", "pssd_gsign", "pssd_gsplit", "pssd_test_fault"]
+           "pssd_test_krylov", "pssd_gsign", "pssd_gsplit", "pssd_test_fault",
+           "pssd_timing_event_count"]
 NOALLOC_MAX_N = 128
 MAX_N = 65535                 # PSSD_MAX_N: largest supported order
 
@@ -134,6 +135,8 @@ def lib():
                                     ctypes.POINTER(Info)]
     L.pssd_device_alloc_count.argtypes = []
     L.pssd_device_alloc_count.restype = ctypes.c_longlong
+    L.pssd_timing_event_count.argtypes = []
+    L.pssd_timing_event_count.restype = ctypes.c_longlong
     L.pssd_launch_count_phases.argtypes = [vp, ctypes.c_int]
     L.pssd_test_krylov.argtypes = [vp, ctypes.c_int, ctypes.c_int, vp, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                    ctypes.c_ulonglong, ctypes.c_int, vp, vp]
@@ -148,6 +151,11 @@ def lib():
 def device_alloc_count() -> int:
     """Device allocations (cudaMalloc calls) the library has made in this process."""
     return int(lib().pssd_device_alloc_count())
+
+
+def timing_event_count() -> int:
+    """CUDA events the library has made for profiling in this process."""
+    return int(lib().pssd_timing_event_count())
 
 
 PHASES = ["other", "front", "bounds", "sign", "split", "shift", "node_sign", "node_split", "assemble", "leaf",

@@ -49,7 +49,10 @@ struct Chunk { char *base; size_t cap; size_t off; bool owned; };   // owned: al
 
 std::atomic<long long> g_device_allocs{0};   // device allocations (cudaMalloc) made by the library
 
-struct ProfEvent { cudaEvent_t a, b; int kind; double flops, bytes; };
+std::atomic<long long> g_timing_events{0};   // events made for profiling
+
+// owner: the handle whose pool the events come from and go back to
+struct ProfEvent { cudaEvent_t a, b; int kind; double flops, bytes; pssd_handle_s *owner; };
 
 }  // namespace
 
@@ -246,6 +249,7 @@ cudaEvent_t get_event(pssd_handle h)
     if (!h->free_events.empty()) { cudaEvent_t e = h->free_events.back(); h->free_events.pop_back(); return e; }
     cudaEvent_t e;
     cuda_check(h, cudaEventCreate(&e), "cudaEventCreate");
+    g_timing_events.fetch_add(1, std::memory_order_relaxed);
     return e;
 }
 
@@ -261,7 +265,7 @@ struct Timed {
     }
     ~Timed()
     {
-        if (h->prof) { cudaEventRecord(b, st); h->events.push_back({a, b, kind, flops, bytes}); }
+        if (h->prof) { cudaEventRecord(b, st); h->events.push_back({a, b, kind, flops, bytes, h}); }
     }
 };
 
@@ -294,8 +298,8 @@ void prof_collect(pssd_handle h)
         h->prof_flops[e.kind] += e.flops;
         h->prof_bytes[e.kind] += e.bytes;
         h->prof_count[e.kind] += 1;
-        h->free_events.push_back(e.a);
-        h->free_events.push_back(e.b);
+        e.owner->free_events.push_back(e.a);
+        e.owner->free_events.push_back(e.b);
     }
     h->events.clear();
 }
@@ -2570,6 +2574,8 @@ long long pssd_launch_count(pssd_handle h) { return h ? g_launches.load() : -1; 
 
 // process-wide number of device allocations (cudaMalloc calls) the library has made
 long long pssd_device_alloc_count(void) { return g_device_allocs.load(); }
+
+long long pssd_timing_event_count(void) { return g_timing_events.load(); }
 
 // the launch count by phase (PSSD_PHASE_* = PH_*)
 int pssd_launch_count_phases(long long *counts, int n)

@@ -131,3 +131,18 @@ def test_helpers_keep_little_between_calls(P):
         h.close()
         kept.append(torch.cuda.mem_get_info()[0] - before)
     assert kept[1] - kept[0] <= 3 * 1024 * MIB + 64 * MIB, kept
+
+
+def test_profiled_calls_reuse_their_events(P):
+    """The timing events of the second halves go back to the pools they came from: ten more calls make fewer events
+    than the first one did."""
+    H = _H(200)
+    h = P.Handle()
+    h.profile(True)
+    n0 = P.timing_event_count()
+    P.eig(H, handle=h)
+    n1 = P.timing_event_count()
+    for _ in range(10):
+        P.eig(H, handle=h)
+    assert P.timing_event_count() - n1 < n1 - n0
+    h.close()
