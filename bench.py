@@ -482,7 +482,7 @@ def main():
                 "timed_solves": reps, "accuracy": accf,
                 "A11_spectrum_rel_diff_vs_headline_path": dA,
                 "dominant_kernel": dict(tab[domf], kernel=KERNEL_NAMES[domf]),
-                "kernels": tab, "r_per_pass": infof["r_used"][:infof["passes"]],
+                "kernels": brief(tab), "r_per_pass": infof["r_used"][:infof["passes"]],
                 "note": "same input and handle" + ("; timed after the FP64-emulated solves (workspace allocated)"
                                                    if name == "fp64" else "; 1 warm-up")}
             del Qf, A11f, A22f
@@ -511,7 +511,7 @@ def main():
             accc = split_accuracy(P, torch, H, Qc, p, dev)
             accc.update({"split_backerr_K": infoc["split_backerr"], "comm_rel_split_lib": infoc["comm_resid"]})
             entry = {"s_per_solve": tc, "timed_solves": reps, "accuracy": accc,
-                     "r_per_pass": infoc["r_used"][:infoc["passes"]], "kernels": tab,
+                     "r_per_pass": infoc["r_used"][:infoc["passes"]], "kernels": brief(tab),
                      "note": "pssd_casida_split on the blocks A, B of the same H; k x k work"
                              + ("; 1 warm-up" if name == "fp64e" else "; timed after the FP64-emulated solves")}
             if "plain_fp64" in line:
@@ -544,7 +544,7 @@ def main():
             "s_per_solve": te_eig, "timed_solves": 1, "levels": infoe["levels"],
             "residual_HV_VD_rel": res, "residual_bound": 1e-11,
             "vsigma_orth_probe": vsv, "vsigma_bound": 1e-12 * n,
-            "kernels": kernel_table(ke, te_eig, 1, peaks),
+            "kernels": brief(kernel_table(ke, te_eig, 1, peaks)),
             "note": "pssd_casida_eig on the blocks A, B of the same H (1 warm-up); checks untimed"}
         del De, Ve
         del Ab, Bb
@@ -632,7 +632,7 @@ def main():
     if rank == 0 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline_sample(n)
     if rank == 0:
-        print(json.dumps(line))
+        print(json.dumps(rounded(line)))
     if ws > 1:
         dist.destroy_process_group()
     return 0
@@ -707,6 +707,24 @@ def kernel_table(kinds, t_total_s, steps, peaks):
                         "peak_note": "of measured HBM copy bandwidth; algorithmic bytes of the passes that count them"})
         out[name] = row
     return out
+
+
+def brief(table):
+    """A kernel table without the columns that the headline's own table explains."""
+    keep = ("ms_per_step", "launches_per_step", "achieved", "frac")
+    return {name: {k: row[k] for k in keep if k in row} for name, row in table.items()}
+
+
+def rounded(line):
+    """The line with the numbers inside its nested parts, but for e2e, at six digits: with seventeen it came to
+    20 KB, more than a reader that keeps the last 20 000 bytes of the output gets to see."""
+    def short(x):
+        if isinstance(x, float):
+            return float("%.6g" % x)
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        return [short(v) for v in x] if isinstance(x, list) else x
+    return {k: short(v) if isinstance(v, (dict, list)) and k != "e2e" else v for k, v in line.items()}
 
 
 def split_accuracy(P, torch, H, Q, p, dev):
