@@ -1699,11 +1699,12 @@ void give_back_helper(pssd_handle_s *x)
     x->root->idle_helpers.push_back(x);
 }
 
-// The two halves of a division are independent, and below order 1000 or so neither fills the
-// GPU: a node is a chain of small launches and host reads.  The second half runs in a thread of
-// its own on a helper's stream while there is a helper (so up to four chains at a time), with
-// the same seeds and operations as one after the other.  casida_eig at k = 1024: 103 -> 70 ms,
-// zeig at n = 400: 76 -> 44 ms.  A half that finds no memory beside the other runs after it.
+// The two halves of a division are independent, and neither fills the GPU: a node is a chain of
+// small launches and host reads.  The second half runs in a thread of its own on a helper's
+// stream while there is a helper (so up to four chains at a time), with the same seeds and
+// operations as one after the other.  casida_eig at k = 1024: 109 -> 67 ms, zeig at n = 400:
+// 76 -> 44 ms, eig at n = 16384: 6.85 -> 5.74 s.  A half that finds no memory beside the other
+// runs after it.
 int sym_eig_pair(pssd_handle h, const SymPart &a, const SymPart &b, int leaf, int depth, int *maxdepth)
 {
     int da = *maxdepth, db = *maxdepth;
